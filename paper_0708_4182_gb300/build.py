@@ -18,7 +18,8 @@ CSRC = os.path.join(PKG, "csrc")
 BUILD = os.path.join(PKG, "_build")
 LIB = os.path.join(BUILD, "liblbm_ewod.so")
 SOURCES = [os.path.join(CSRC, "lbm_ewod.cu")]
-DEPS = SOURCES + [os.path.join(CSRC, "lbm_step.cuh"), os.path.join(ROOT, "include", "lbm_ewod.h")]
+DEPS = SOURCES + [os.path.join(CSRC, "lbm_step.cuh"), os.path.join(CSRC, "lbm_resident.cuh"),
+                  os.path.join(ROOT, "include", "lbm_ewod.h")]
 UNET_LIB = os.path.join(BUILD, "libunet_bf16.so")
 UNET_SOURCES = [os.path.join(CSRC, "unet_bf16.cu")]
 UNET_DEPS = UNET_SOURCES + [os.path.join(ROOT, "include", "unet_bf16.h")]

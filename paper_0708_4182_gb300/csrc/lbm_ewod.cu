@@ -10,14 +10,17 @@
 //             one scratch record for lbm_observables
 //   status    int error flag raised by bounded device-side waits that gave up
 //   staging   bounded buffer for host <-> device transfers of FP64 populations
+//   exch      exchange records of the resident steps (domains that fit on the chip)
 #include "lbm_ewod.h"
 #include "lbm_step.cuh"
+#include "lbm_resident.cuh"
 
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <utility>
 #include <mutex>
 #include <new>
 #include <algorithm>
@@ -35,10 +38,22 @@ size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
 int pitch_of(int nx) { return (nx + 31) / 32 * 32; }
 
+// How a domain runs in the resident kernel (lbm_resident.cuh): tx x ty tiles,
+// a halo of 2 k nodes exchanged every k steps, nt threads per CTA with j rows
+// per warp at most. tx = 0: it does not (too large).
+struct ResPlan {
+    int tx = 0, ty = 0, k = 0, j = 0, nt = 0;
+    int edge_cap = 0;  // records per tile and value group
+    size_t smem = 0;
+    double cycles = 0.0;  // estimated SM cycles per step
+    int tiles() const { return tx * ty; }
+};
+
 struct Layout {
-    size_t off_a, off_b, off_mask, off_partials, off_ring, off_status, off_staging, total;
-    size_t pops_bytes, staging_bytes;
+    size_t off_a, off_b, off_mask, off_partials, off_ring, off_status, off_staging, off_exch, total;
+    size_t pops_bytes, staging_bytes, exch_bytes;
     int max_ctas;
+    ResPlan res;
 };
 
 bool params_valid(const lbm_params* p, const char** why)
@@ -71,7 +86,82 @@ bool params_valid(const lbm_params* p, const char** why)
 // CTAs across a domain of nx columns (strips of strip_cols(storage) columns)
 int ctas_x(int nx, int storage) { return (nx + strip_cols(storage) - 1) / strip_cols(storage); }
 
-Layout layout_of(const lbm_params* p)
+constexpr int kResSms = 152;                     // SMs of a GB300
+constexpr size_t kResSmemCta = 227 * 1024;       // shared memory of a CTA at most
+constexpr size_t kResSmemSm = 228 * 1024;        // of an SM; a CTA takes 1 KB of it and its static part as well
+
+size_t res_smem(int storage, int rows, int nhalo)
+{
+    return storage == LBM_FP32       ? res_smem_bytes<kF32>(rows, nhalo)
+           : storage == LBM_FP32_DEV ? res_smem_bytes<kF32Dev>(rows, nhalo)
+                                     : res_smem_bytes<kF16Dev>(rows, nhalo);
+}
+
+// Estimated cycles per step of tiles of w x h nodes with `per_sm` of them on
+// the busiest SM: a step (two barriers) costs about 300 cycles and the larger
+// of the latency of one warp's rows (900, or 1400 a row when there are
+// several) and the SM's issue slots (75 a row); an exchange costs about 1800,
+// once every k steps. Measured (cycles a step): 1024x256 in 280 tiles 6700 in
+// FP32 and 7800 in FP32 deviations (estimated 7200), 1024x512 in 455 tiles
+// 10600 (11550), 128x64 in 128 tiles at k = 4 1950 (1800).
+bool res_try(int storage, bool t1, int w, int h, int k, int per_sm, ResPlan* r)
+{
+    const int H = h + 4 * k, W = w + 4 * k, nhalo = W * H - w * h;
+    if (W > kResP) return false;
+    const size_t smem = res_smem(storage, H, nhalo);
+    if (smem > kResSmemCta || size_t(per_sm) * (smem + 1280) > kResSmemSm) return false;
+    r->cycles = -1.0;
+    for (int j = 1; j <= (t1 ? kResMaxRows : 2); ++j) {
+        const int nw = (H - 2 + j - 1) / j;
+        // registers: 56 a thread (j <= 2) or 64, in units of 8
+        if (nw * 32 > res_max_threads(j) || per_sm * nw * 32 * (j <= 2 ? 56 : 64) > 65536) continue;
+        double c = 1800.0;
+        for (int m = 0; m < k; ++m) {
+            const int rows = H - 2 - 4 * m;
+            c += 300.0 + std::max(j == 1 ? 900.0 : 1400.0 * ((rows + nw - 1) / nw), 75.0 * rows * per_sm);
+        }
+        c /= k;
+        if (r->cycles < 0.0 || c < r->cycles) {
+            r->cycles = c;
+            r->j = j;
+            r->nt = 32 * nw;
+            r->k = k;
+            r->smem = smem;
+        }
+    }
+    return r->cycles >= 0.0;
+}
+
+// The tiling with the fewest estimated cycles per step.
+ResPlan res_plan(int nx, int ny, int storage, bool t1)
+{
+    ResPlan best;
+    const int most = 4 * kResSms;
+    for (int k = 1; k <= 4; k *= 2) {
+        const int wmax = kResP - 4 * k, first = (nx + wmax - 1) / wmax;
+        for (int tx = first; tx <= std::min({nx, most, 2 * first}); ++tx) {
+            const int w = (nx + tx - 1) / tx;
+            if (tx > first && (nx + tx - 2) / (tx - 1) == w) continue;  // no narrower than with tx - 1
+            for (int ty = 1; ty <= std::min(ny, most / tx); ++ty) {
+                const int h = (ny + ty - 1) / ty;
+                if (ty > 1 && (ny + ty - 2) / (ty - 1) == h) continue;
+                ResPlan r;
+                if (!res_try(storage, t1, w, h, k, (tx * ty + kResSms - 1) / kResSms, &r)) continue;
+                if (best.tx && r.cycles >= best.cycles) continue;
+                r.tx = tx;
+                r.ty = ty;
+                for (int a = 0; a < 2; ++a)
+                    for (int b = 0; b < 2; ++b)
+                        r.edge_cap = std::max(r.edge_cap, res_edge_nodes(nx / tx + (a && nx % tx), ny / ty + (b && ny % ty), 2 * k));
+                best = r;
+            }
+        }
+    }
+    return best;
+}
+
+// single: a domain of its own, else one of a batch (whose resident steps are the batch's)
+Layout layout_of(const lbm_params* p, bool single)
 {
     Layout L{};
     const int pitch = pitch_of(p->nx);
@@ -88,6 +178,12 @@ Layout layout_of(const lbm_params* p)
     L.staging_bytes = full < kStagingMax ? full : kStagingMax;
     if (L.staging_bytes < size_t(9) * p->nx * sizeof(double)) L.staging_bytes = size_t(9) * p->nx * sizeof(double);
     L.off_staging = o; o = align_up(o + L.staging_bytes, 256);
+    L.off_exch = o;
+    if (single && p->layout == LBM_LAYOUT_AUTO && p->tile_rows == 0) {
+        L.res = res_plan(p->nx, p->ny, p->storage, float(p->tau) == 1.f);
+        L.exch_bytes = size_t(2) * L.res.tiles() * res_records(p->storage) * L.res.edge_cap * sizeof(uint4);
+    }
+    o = align_up(o + L.exch_bytes, 256);
     L.total = o;
     return L;
 }
@@ -710,6 +806,8 @@ struct lbm_ctx {
     // kGraphSteps plain steps as one CUDA graph, one per buffer holding the
     // current state (buffer A, buffer B); built on first use
     cudaGraphExec_t step_graph[2] = {nullptr, nullptr};
+    uint4* exch = nullptr;  // exchange records of the resident kernel (NULL: not used)
+    uint32_t res_tag = 1;   // next unused tag
     ~lbm_ctx()
     {
         for (cudaGraphExec_t e : step_graph)
@@ -909,6 +1007,105 @@ cudaError_t allow_smem()
     return e;
 }
 
+// The resident kernel (one domain or a batch) for j rows per warp.
+template <int ST, bool T1, int J> const void* resident_inst(bool batch)
+{
+    return batch ? reinterpret_cast<const void*>(&resident_batch_kernel<ST, T1, J>)
+                 : reinterpret_cast<const void*>(&resident_kernel<ST, T1, J>);
+}
+template <int ST> const void* resident_ptr(bool t1, int j, bool batch)
+{
+    if (!t1) return j == 1 ? resident_inst<ST, false, 1>(batch) : resident_inst<ST, false, 2>(batch);
+    return j == 1   ? resident_inst<ST, true, 1>(batch)
+           : j == 2 ? resident_inst<ST, true, 2>(batch)
+                    : resident_inst<ST, true, kResMaxRows>(batch);
+}
+const void* resident_fn(int storage, bool t1, int j, bool batch)
+{
+    switch (storage) {
+    case LBM_FP32_DEV: return resident_ptr<kF32Dev>(t1, j, batch);
+    case LBM_FP16_DEV: return resident_ptr<kF16Dev>(t1, j, batch);
+    case LBM_BF16_DEV: return resident_ptr<kBF16Dev>(t1, j, batch);
+    default: return resident_ptr<kF32>(t1, j, batch);
+    }
+}
+
+// Allow the launch shape of a plan; false if its CTAs would not be resident
+// together on this device.
+bool resident_fits(const void* fn, const ResPlan& r, int ctas, int sm_count)
+{
+    int per_sm = 0;
+    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, int(r.smem)) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, r.nt, r.smem) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return (long long)per_sm * sm_count >= ctas;
+}
+
+// The tags of n more steps: the first of them. Tags of one exchange buffer
+// (bytes at exch) are not used twice; near the end of their 32 bits the
+// buffer is cleared and they start again.
+lbm_status take_tags(uint32_t* next, int n, uint4* exch, size_t bytes, cudaStream_t st, uint32_t* first)
+{
+    if (*next > 0xffffffffu - uint32_t(n)) {
+        if (cudaMemsetAsync(exch, 0, bytes, st) != cudaSuccess) return LBM_ECUDA;
+        *next = 1;
+    }
+    *first = *next;
+    *next += uint32_t(n);
+    return LBM_OK;
+}
+
+bool capturing(cudaStream_t st)
+{
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cs) != cudaSuccess) {
+        cudaGetLastError();
+        return true;
+    }
+    return cs != cudaStreamCaptureStatusNone;
+}
+
+// Steps per resident launch at most: about a millisecond or two, so that
+// other streams' work gets its turn.
+constexpr int kResChunk = 1024;
+// Fewer steps are launched one by one: a resident launch loads and stores the
+// state once more. Measured (us for 2 and 3 steps, resident / one by one):
+// 128x64 8.6 and 9.8 / 16.7 and 24.8; 1024x512 30 and 36 / 29 and 43.
+constexpr int kResMinSteps = 2;
+
+// nsteps plain steps of a domain that fits on the chip. *done = false if this
+// device cannot hold the launch right now (the caller steps one by one).
+lbm_status resident_steps(lbm_ctx* c, int64_t nsteps, bool* done)
+{
+    const ResPlan& r = c->L.res;
+    const void* fn = resident_fn(c->prm.storage, c->ph.tau == 1.f, r.j, false);
+    *done = true;
+    while (nsteps > 0) {
+        int n = int(std::min<int64_t>(nsteps, kResChunk));
+        const float* in = c->cur;
+        float* out = c->nxt;
+        int tx = r.tx, ty = r.ty, k = r.k, cap = r.edge_cap, stride = int(c->L.exch_bytes / 2 / sizeof(uint4));
+        uint32_t tag = 0;
+        lbm_status s = take_tags(&c->res_tag, n, c->exch, c->L.exch_bytes, c->stream, &tag);
+        if (s) return fail(c, s, "exchange buffer clear");
+        void* args[] = {&in, &out, &c->g, &c->ph, &tx, &ty, &k, &c->exch, &stride, &cap, &tag, &n, &c->status};
+        const cudaError_t e = cudaLaunchCooperativeKernel(fn, dim3(r.tiles()), dim3(r.nt), args, r.smem, c->stream);
+        if (e == cudaErrorCooperativeLaunchTooLarge) {
+            cudaGetLastError();
+            c->exch = nullptr;
+            *done = false;
+            return LBM_OK;
+        }
+        if ((s = check_cuda(c, e, "resident steps launch"))) return s;
+        c->t += n;
+        std::swap(c->cur, c->nxt);
+        nsteps -= n;
+    }
+    return LBM_OK;
+}
+
 // Convert the plain f* in c->cur to the context's deviation form (into the
 // spare buffer, which becomes current). No-op for plain storage.
 lbm_status plain_to_storage(lbm_ctx* c)
@@ -982,18 +1179,18 @@ size_t lbm_workspace_bytes(const lbm_params* p)
 {
     const char* why;
     if (!params_valid(p, &why)) return 0;
-    return layout_of(p).total;
+    return layout_of(p, true).total;
 }
 
-lbm_status lbm_create(const lbm_params* p, void* d_workspace, size_t bytes, void* cuda_stream,
-                      lbm_ctx** out)
+static lbm_status create_ctx(const lbm_params* p, void* d_workspace, size_t bytes, void* cuda_stream, bool single,
+                             lbm_ctx** out)
 {
     if (!out) return LBM_EINVAL;
     *out = nullptr;
     const char* why = "";
     if (!params_valid(p, &why)) return LBM_EINVAL;
     if (!d_workspace || (reinterpret_cast<uintptr_t>(d_workspace) & 255u)) return LBM_EINVAL;
-    Layout L = layout_of(p);
+    Layout L = layout_of(p, single);
     if (bytes < L.total) return LBM_ENOMEM;
     lbm_ctx* c = new (std::nothrow) lbm_ctx;
     if (!c) return LBM_ENOMEM;
@@ -1035,8 +1232,21 @@ lbm_status lbm_create(const lbm_params* p, void* d_workspace, size_t bytes, void
         p->tile_rows ? p->tile_rows : auto_tile_rows(p->nx, p->ny, p->storage, c->sm_count, c->pair);
     c->grid = dim3(ctas_x(p->nx, p->storage), (p->ny + c->g.tile_rows - 1) / c->g.tile_rows);
     c->ph = make_phys(*p);
+    if (L.exch_bytes && resident_fits(resident_fn(p->storage, c->ph.tau == 1.f, L.res.j, false), L.res, L.res.tiles(), c->sm_count)) {
+        c->exch = reinterpret_cast<uint4*>(c->ws + L.off_exch);
+        if (cudaMemsetAsync(c->exch, 0, L.exch_bytes, c->stream) != cudaSuccess) {
+            cudaGetLastError();
+            delete c;
+            return LBM_ECUDA;
+        }
+    }
     *out = c;
     return LBM_OK;
+}
+
+lbm_status lbm_create(const lbm_params* p, void* d_workspace, size_t bytes, void* cuda_stream, lbm_ctx** out)
+{
+    return create_ctx(p, d_workspace, bytes, cuda_stream, true, out);
 }
 
 lbm_status lbm_set_geometry(lbm_ctx* c, const uint8_t* solid, int on_device)
@@ -1239,7 +1449,21 @@ lbm_status lbm_step(lbm_ctx* c, int64_t nsteps)
     if (s) return s;
     if (nsteps < 0) return fail(c, LBM_EINVAL, "nsteps must be >= 0");
     const int K = c->prm.obs_every;
+    const bool capture = c->exch && capturing(c->stream);  // a captured call keeps its launches
     for (int64_t k = 0; k < nsteps; ++k) {
+        if (c->exch && !capture) {
+            // plain steps up to the next observed one: on the chip from
+            // kResMinSteps on
+            const int64_t run = K == 0 ? nsteps - k : (c->t % K == 0 ? 0 : std::min<int64_t>(nsteps - k, K - c->t % K));
+            if (run >= kResMinSteps) {
+                bool done;
+                const int64_t t0 = c->t;
+                if ((s = resident_steps(c, run, &done))) return s;
+                k += c->t - t0 - 1;
+                if (done || c->t != t0) continue;
+                ++k;
+            }
+        }
         // whole graphs of plain steps while no fused-observables step falls inside
         if (nsteps - k >= kGraphSteps && (K == 0 || (c->t % K != 0 && c->t / K == (c->t + kGraphSteps - 1) / K))) {
             cudaGraphExec_t exec;
@@ -1521,6 +1745,20 @@ struct lbm_batch {
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
     int graph_ntiles = -1, graph_grid = -1;
+    // resident steps: the active domains in groups that fit on the chip, each
+    // one launch of CTAs first .. first + ctas - 1 of the CTA table
+    struct Group { ResPlan plan; int first, ctas; };
+    bool res_allowed = false;            // automatic layout and tiling throughout
+    std::vector<Group> groups;
+    double res_us = 0.0, res_us_once = 0.0, walk_us = 0.0;  // estimated time per step, per call; of the tile walk per step
+    bool groups_dirty = true;
+    uint4* exch = nullptr;
+    size_t exch_bytes = 0;
+    uint32_t res_tag = 1;
+    int4* d_shape = nullptr;             // per domain: tx, ty, first CTA of its group's launch
+    int2* d_ctas = nullptr;              // (domain, tile) of every CTA
+    std::vector<int4> h_shape;
+    std::vector<int2> h_ctas;
     char err[512] = {0};
 };
 
@@ -1543,9 +1781,13 @@ lbm_status bcheck(lbm_batch* b, cudaError_t e, const char* what)
     return bfail(b, LBM_ECUDA, "%s: %s", what, cudaGetErrorString(e));
 }
 
+constexpr int kResCtas = 4 * kResSms;       // CTAs of a resident launch at most
+constexpr int kResEdgeNodes = 1 << 18;      // their published nodes at most (25 MB of exchange records)
+
 struct BatchLayout {
     std::vector<size_t> off;  // per-domain workspace offsets
     size_t off_dom, off_tiles, off_status, off_rec, off_ptrs, off_nctas, off_invnx, off_step, off_want, total;
+    size_t off_shape, off_ctas, off_exch, exch_bytes;
     int max_tiles;
 };
 
@@ -1559,7 +1801,7 @@ bool batch_layout(const lbm_params* p, int count, BatchLayout* L, const char** w
         if (!params_valid(&p[i], why)) return false;
         if (p[i].storage != p[0].storage) { *why = "all domains of a batch share one storage form"; return false; }
         L->off[i] = o;
-        o = align_up(o + layout_of(&p[i]).total, 256);
+        o = align_up(o + layout_of(&p[i], false).total, 256);
         L->max_tiles += ctas_x(p[i].nx, p[i].storage) * ((p[i].ny + 3) / 4);
     }
     L->off_dom = o; o = align_up(o + count * sizeof(DomainDev), 256);
@@ -1571,6 +1813,10 @@ bool batch_layout(const lbm_params* p, int count, BatchLayout* L, const char** w
     L->off_invnx = o; o = align_up(o + count * sizeof(double), 256);
     L->off_step = o; o = align_up(o + count * sizeof(long long), 256);
     L->off_want = o; o = align_up(o + count, 256);
+    L->off_shape = o; o = align_up(o + count * sizeof(int4), 256);
+    L->off_ctas = o; o = align_up(o + size_t(count) * kResCtas * sizeof(int2), 256);
+    L->exch_bytes = size_t(2) * res_records(p[0].storage) * kResEdgeNodes * sizeof(uint4);
+    L->off_exch = o; o = align_up(o + L->exch_bytes, 256);
     L->total = o;
     return true;
 }
@@ -1738,6 +1984,152 @@ lbm_status batch_graph(lbm_batch* b)
     return LBM_OK;
 }
 
+// Group the active domains for resident steps (largest first into the first
+// group with room), for the tile height and exchange interval whose groups
+// take the fewest estimated cycles together. groups stays empty where a
+// domain does not fit on the chip.
+void plan_groups(lbm_batch* b)
+{
+    b->groups.clear();
+    b->groups_dirty = false;
+    std::vector<int> order;
+    long long nodes = 0;
+    for (int d = 0; d < b->count; ++d)
+        if (b->active[d]) {
+            order.push_back(d);
+            nodes += (long long)b->ctx[d]->g.nx * b->ctx[d]->g.ny;
+        }
+    std::sort(order.begin(), order.end(), [&](int x, int y) {
+        return (long long)b->ctx[x]->g.nx * b->ctx[x]->g.ny > (long long)b->ctx[y]->g.nx * b->ctx[y]->g.ny;
+    });
+    // the tile walk: about 12 us of latency and 80 GLUPS (measured: 64 channels
+    // of 256x64 28 us, 256 uneven channels 81.7 GLUPS in FP32)
+    b->walk_us = 12.0 + double(nodes) / 80e3;
+    struct Trial { int w = 0, h = 0, ctas = 0, edge = 0, hmax = 0; std::vector<int> doms; };
+    static const int heights[] = {4, 8, 12, 16, 20, 24, 28, 32, 40, 48, 56, 64, 72, 80, 96, 112, 128, 144};
+    double best = -1.0;
+    std::vector<Trial> pick;
+    std::vector<ResPlan> plans;
+    for (int k = 1; k <= 4; k *= 2) {
+        const int wmax = kResP - 4 * k;
+        for (int hmax : heights) {
+            // CTAs of this height that fit on an SM
+            ResPlan r;
+            int per_sm = 0;
+            while (per_sm < 4 && res_try(b->storage, b->tau1, wmax, hmax, k, per_sm + 1, &r)) ++per_sm;
+            if (!per_sm) continue;
+            std::vector<Trial> trial;
+            bool ok = true;
+            for (int d : order) {
+                const Geom& g = b->ctx[d]->g;
+                const int tx = (g.nx + wmax - 1) / wmax, ty = (g.ny + hmax - 1) / hmax;
+                const int w = (g.nx + tx - 1) / tx, h = (g.ny + ty - 1) / ty;
+                const int edge = res_edge_nodes(w, h, 2 * k);
+                if (tx * ty > per_sm * kResSms) { ok = false; break; }
+                size_t i = 0;
+                while (i < trial.size() && (trial[i].ctas + tx * ty > per_sm * kResSms ||
+                                            (trial[i].ctas + tx * ty) * std::max(trial[i].edge, edge) > kResEdgeNodes))
+                    ++i;
+                if (i == trial.size()) trial.emplace_back();
+                Trial& t = trial[i];
+                t.ctas += tx * ty;
+                t.w = std::max(t.w, w);
+                t.h = std::max(t.h, h);
+                t.edge = std::max(t.edge, edge);
+                t.hmax = hmax;
+                t.doms.push_back(d);
+            }
+            if (!ok) continue;
+            double cost = 0.0;
+            std::vector<ResPlan> rs;
+            for (const Trial& t : trial) {
+                if (!res_try(b->storage, b->tau1, t.w, t.h, k, (t.ctas + kResSms - 1) / kResSms, &r)) { ok = false; break; }
+                r.edge_cap = t.edge;
+                cost += r.cycles;
+                rs.push_back(r);
+            }
+            if (ok && (best < 0.0 || cost < best)) {
+                best = cost;
+                pick = trial;
+                plans = rs;
+            }
+        }
+    }
+    if (best < 0.0) return;
+    b->h_ctas.clear();
+    for (size_t i = 0; i < pick.size(); ++i) {
+        lbm_batch::Group gr{plans[i], int(b->h_ctas.size()), pick[i].ctas};
+        int first = 0;
+        for (int d : pick[i].doms) {
+            const Geom& g = b->ctx[d]->g;
+            const int wmax = kResP - 4 * gr.plan.k;
+            const int tx = (g.nx + wmax - 1) / wmax, ty = (g.ny + pick[i].hmax - 1) / pick[i].hmax;
+            b->h_shape[d] = make_int4(tx, ty, first, 0);
+            for (int t = 0; t < tx * ty; ++t) b->h_ctas.push_back(make_int2(d, t));
+            first += tx * ty;
+        }
+        gr.ctas = first;
+        if (!resident_fits(resident_fn(b->storage, b->tau1, gr.plan.j, true), gr.plan, gr.ctas, b->sm_count)) {
+            b->groups.clear();
+            return;
+        }
+        b->groups.push_back(gr);
+    }
+    b->res_us = best / 1900.0;  // at 1.9 GHz
+    // a launch, and the state in and out once
+    b->res_us_once = 8.0 * double(b->groups.size()) + double(nodes) * 72.0 / 4e6;
+}
+
+// nsteps plain steps of the active domains, group after group. *done = false
+// where they are better or only possible by the tile walk.
+lbm_status resident_batch_steps(lbm_batch* b, int64_t nsteps, bool* done)
+{
+    *done = false;
+    if (!b->res_allowed || capturing(b->stream)) return LBM_OK;
+    lbm_status s;
+    if (b->groups_dirty) {
+        plan_groups(b);
+        if (!b->groups.empty()) {
+            if ((s = bcheck(b, cudaMemcpyAsync(b->d_shape, b->h_shape.data(), b->count * sizeof(int4),
+                                               cudaMemcpyHostToDevice, b->stream), "tiling upload")) ||
+                (s = bcheck(b, cudaMemcpyAsync(b->d_ctas, b->h_ctas.data(), b->h_ctas.size() * sizeof(int2),
+                                               cudaMemcpyHostToDevice, b->stream), "CTA table upload")))
+                return s;
+        }
+    }
+    if (b->groups.empty() || b->res_us * double(nsteps) + b->res_us_once >= b->walk_us * double(nsteps)) return LBM_OK;
+    int launches = 0;
+    for (const lbm_batch::Group& gr : b->groups) {
+        const void* fn = resident_fn(b->storage, b->tau1, gr.plan.j, true);
+        const int2* ctas = b->d_ctas + gr.first;
+        int k = gr.plan.k, cap = gr.plan.edge_cap, stride = gr.ctas * res_records(b->storage) * cap;
+        launches = 0;
+        for (int64_t left = nsteps; left > 0; ++launches) {
+            int n = int(std::min<int64_t>(left, kResChunk)), parity = launches & 1;
+            uint32_t tag = 0;
+            if ((s = take_tags(&b->res_tag, n, b->exch, b->exch_bytes, b->stream, &tag)))
+                return bfail(b, s, "exchange buffer clear");
+            void* args[] = {&b->d_dom, &b->d_shape, &ctas, &parity, &k, &b->exch, &stride, &cap, &tag, &n, &b->d_status};
+            const cudaError_t e = cudaLaunchCooperativeKernel(fn, dim3(gr.ctas), dim3(gr.plan.nt), args, gr.plan.smem, b->stream);
+            if (e == cudaErrorCooperativeLaunchTooLarge && launches == 0 && &gr == &b->groups.front()) {
+                cudaGetLastError();
+                b->res_allowed = false;
+                return LBM_OK;
+            }
+            if ((s = bcheck(b, e, "resident steps launch"))) return s;
+            left -= n;
+        }
+    }
+    for (int d = 0; d < b->count; ++d) {
+        if (!b->active[d]) continue;
+        lbm_ctx* c = b->ctx[d];
+        c->t += nsteps;
+        if (launches & 1) std::swap(c->cur, c->nxt);
+    }
+    *done = true;
+    return LBM_OK;
+}
+
 lbm_status batch_ready(lbm_batch* b)
 {
     if (!b) return LBM_EINVAL;
@@ -1827,8 +2219,8 @@ lbm_status lbm_batch_create(const lbm_params* params, int32_t count, void* d_wor
     b->active.assign(count, 1);
     b->h_dom.resize(count);
     for (int d = 0; d < count; ++d) {
-        const size_t need = layout_of(&params[d]).total;
-        lbm_status s = lbm_create(&params[d], ws + L.off[d], need, cuda_stream, &b->ctx[d]);
+        const size_t need = layout_of(&params[d], false).total;
+        lbm_status s = create_ctx(&params[d], ws + L.off[d], need, cuda_stream, false, &b->ctx[d]);
         if (s) {
             for (int e = 0; e < d; ++e) lbm_destroy(b->ctx[e]);
             delete b;
@@ -1846,7 +2238,15 @@ lbm_status lbm_batch_create(const lbm_params* params, int32_t count, void* d_wor
     b->d_step = reinterpret_cast<long long*>(ws + L.off_step);
     b->d_want = ws + L.off_want;
     b->max_tiles = L.max_tiles;
-    cudaError_t e = cudaSuccess;
+    b->d_shape = reinterpret_cast<int4*>(ws + L.off_shape);
+    b->d_ctas = reinterpret_cast<int2*>(ws + L.off_ctas);
+    b->exch = reinterpret_cast<uint4*>(ws + L.off_exch);
+    b->exch_bytes = L.exch_bytes;
+    b->h_shape.resize(count);
+    b->res_allowed = true;
+    for (int d = 0; d < count; ++d)
+        if (params[d].layout != LBM_LAYOUT_AUTO || params[d].tile_rows != 0) b->res_allowed = false;
+    cudaError_t e = cudaMemsetAsync(b->exch, 0, b->exch_bytes, b->stream);
     for (int d = 0; d < count; ++d)
         if (b->ctx[d]->ph.tau != 1.f) b->tau1 = false;
     // Thread layout (32-bit forms), by the rule of a single domain applied to
@@ -1899,6 +2299,7 @@ lbm_status lbm_batch_set_active(lbm_batch* b, const uint8_t* active)
     if (!b || !active) return LBM_EINVAL;
     for (int d = 0; d < b->count; ++d) b->active[d] = active[d] ? 1 : 0;
     b->tiles_dirty = true;
+    b->groups_dirty = true;
     return LBM_OK;
 }
 
@@ -1921,6 +2322,8 @@ lbm_status lbm_batch_step(lbm_batch* b, int64_t nsteps)
     if (nsteps == 0) return LBM_OK;
     if ((s = upload_tables(b, false))) return s;
     if (b->ntiles == 0) return LBM_OK;
+    bool done;
+    if ((s = resident_batch_steps(b, nsteps, &done)) || done) return s;
     if ((s = batch_graph(b))) return s;
     for (int64_t k = 0; k + 1 < nsteps; k += 2)
         if ((s = bcheck(b, cudaGraphLaunch(b->exec, b->stream), "graph launch"))) return s;
@@ -2018,6 +2421,7 @@ lbm_status lbm_batch_run_to_steady(lbm_batch* b, double rel_tol, int64_t check_e
         }
         if (changed) {
             b->tiles_dirty = true;
+            b->groups_dirty = true;
             retile();
         }
     }
@@ -2025,6 +2429,7 @@ lbm_status lbm_batch_run_to_steady(lbm_batch* b, double rel_tol, int64_t check_e
     b->active = start_active;
     b->tile_rows = rows_start;
     b->tiles_dirty = true;
+    b->groups_dirty = true;
     if (first_nan >= 0) return bfail(b, LBM_ENAN, "domain %d became non-finite", first_nan);
     for (int d = 0; d < b->count; ++d)
         if (start_active[d] && steps_to_steady[d] < 0) return bfail(b, LBM_ENOTCONV, "domain %d not steady", d);
@@ -2041,6 +2446,8 @@ lbm_status lbm_batch_autotune(lbm_batch* b, const int32_t* candidates, int32_t n
     if ((s = bcheck(b, cudaEventCreate(&e0), "event")) || (s = bcheck(b, cudaEventCreate(&e1), "event"))) return s;
     double best = 1e300;
     int32_t pick = b->tile_rows;
+    const bool res_allowed = b->res_allowed;
+    b->res_allowed = false;  // the heights are those of the tile walk
     for (int i = 0; i < n; ++i) {
         if ((s = lbm_batch_set_tile_rows(b, candidates[i]))) break;
         if ((s = lbm_batch_step(b, 2))) break;  // warm-up (and graph build)
@@ -2059,6 +2466,7 @@ lbm_status lbm_batch_autotune(lbm_batch* b, const int32_t* candidates, int32_t n
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
+    b->res_allowed = res_allowed;
     if (s) return s;
     *chosen = pick;
     if ((s = lbm_batch_set_tile_rows(b, pick))) return s;

@@ -482,19 +482,25 @@ __device__ __forceinline__ void wall_electric(uint32_t sb, float psi, float nsgx
 // symmetric, so this is exactly the negated sum); every operation is the
 // two-node kernel's (node_force2) lane for lane. The x and y components go
 // through the paired instructions together (lane x: the x component).
-template <typename N>
-__device__ __forceinline__ float2 node_force(const N& n, const float* pm, const float* pc, const float* pp,
-                                             int t, const Phys& p)
+// psi_sums: the Eq. 5 sum before the factor psi(x), negated.
+__device__ __forceinline__ float2 psi_sums(const float* pm, const float* pc, const float* pp, int t, const Phys& p)
 {
-    const float psi = pc[t];
     // (psi(x+1) - psi(x-1), psi(y+1) - psi(y-1)) on the node's row and column
     const float2 dc = sub2(make_float2(pc[t + 1], pp[t]), make_float2(pc[t - 1], pm[t]));
     // rows y+1 and y-1: right minus left, right plus left
     const float2 pr = make_float2(pp[t + 1], pm[t + 1]), pl = make_float2(pp[t - 1], pm[t - 1]);
     const float2 dd = sub2(pr, pl), ss = add2(pr, pl);
     // Eq. 5: -sum_a G_a psi(x+e_a) e_a, axis and diagonal links
-    const float2 nsg = fma2(splat(-p.g_axis), dc,
-                            mul2(splat(-p.g_diag), make_float2(__fadd_rn(dd.x, dd.y), __fsub_rn(ss.x, ss.y))));
+    return fma2(splat(-p.g_axis), dc,
+                mul2(splat(-p.g_diag), make_float2(__fadd_rn(dd.x, dd.y), __fsub_rn(ss.x, ss.y))));
+}
+
+template <typename N>
+__device__ __forceinline__ float2 node_force(const N& n, const float* pm, const float* pc, const float* pp,
+                                             int t, const Phys& p)
+{
+    const float psi = pc[t];
+    const float2 nsg = psi_sums(pm, pc, pp, t, p);
     float2 F = mul2(splat(psi), nsg);
     if (n.sb != 0) wall_electric(n.sb, psi, nsg.x, nsg.y, n.rho, p, F.x, F.y);
     // body force on every fluid node
@@ -549,6 +555,39 @@ __device__ __forceinline__ float2 div2(float2 n, float2 nd, float2 r)
     return fma2(e, r, q0);
 }
 
+// Eq. 10 velocity shift, Eq. 3 equilibrium and Eq. 1 relaxation of one node in
+// plain storage under the force F: its post-collision populations fs; rinv is
+// rcp_approx(rho).
+template <bool T1>
+__device__ __forceinline__ void relax_node(const Pulled& n, float2 F, float rinv, const Phys& p, float (&fs)[9])
+{
+    // FP32 care: u' by corrected quotients; the weights w_a rho all derive
+    // from one corrected rho/9 by exact power-of-two scalings, so
+    // sum_a f_eq = rho has no systematic bias (1/9 in FP32 is 7.5e-9 too
+    // large, which would add mass every step); at tau = 1 f* = f_eq.
+    // Lane pairs: (x, y) components, then the directions (1, 2), (3, 4),
+    // (5, 6), (7, 8).
+    const float2 u = div2(fma2(splat(p.tau), F, make_float2(n.jx, n.jy)), splat(-n.rho), splat(rinv));
+    const float om = fmaf(-1.5f, fmaf(u.x, u.x, __fmul_rn(u.y, u.y)), 1.f);
+    const float r9 = div1(n.rho, -9.f, 1.f / 9.f);
+    const float w0r = __fmul_rn(4.f, r9), w2r = __fmul_rn(0.25f, r9);
+    const float2 dg = make_float2(__fadd_rn(u.x, u.y), __fsub_rn(u.y, u.x));  // e5.u, e6.u
+    // f_eq_a = w_a rho (1 + 3 c + 4.5 c^2 - 1.5 u^2) with c = +-(e_a . u):
+    // (-c)(4.5(-c) + 3) = c (4.5 c - 3) exactly
+    const float2 oms = splat(om);
+    auto polyp = [oms](float2 c) { return fma2(c, fma2(splat(4.5f), c, splat(3.f)), oms); };
+    auto polym = [oms](float2 c) { return fma2(c, fma2(splat(4.5f), c, splat(-3.f)), oms); };
+    fs[0] = __fmul_rn(w0r, om);
+    const float2 f12 = mul2(splat(r9), polyp(u)), f34 = mul2(splat(r9), polym(u));
+    const float2 f56 = mul2(splat(w2r), polyp(dg)), f78 = mul2(splat(w2r), polym(dg));
+    fs[1] = f12.x; fs[2] = f12.y; fs[3] = f34.x; fs[4] = f34.y;
+    fs[5] = f56.x; fs[6] = f56.y; fs[7] = f78.x; fs[8] = f78.y;
+    if (!T1 && p.tau != 1.f) {
+#pragma unroll
+        for (int a = 0; a < 9; ++a) fs[a] = fmaf(__fsub_rn(fs[a], n.f[a]), p.inv_tau, n.f[a]);
+    }
+}
+
 // Forces, velocity shift, collision and the mode's epilogue for one fluid node
 // (x, r) in plain storage, whose pulled populations are `n`; psi rows r-1, r,
 // r+1 are pm, pc, pp (indexed by the node's ring column t). Every operation is
@@ -563,33 +602,8 @@ __device__ __forceinline__ void collide_node(const Pulled& n, const float* pm, c
     const float2 F = node_force(n, pm, pc, pp, t, p);
     const float rinv = rcp_approx(n.rho);
     if constexpr (MODE == kStep || MODE == kStepObs) {
-        // Eq. 10 velocity shift, Eq. 3 equilibrium, Eq. 1 relaxation.
-        // FP32 care: u' by corrected quotients; the weights w_a rho all derive
-        // from one corrected rho/9 by exact power-of-two scalings, so
-        // sum_a f_eq = rho has no systematic bias (1/9 in FP32 is 7.5e-9 too
-        // large, which would add mass every step); at tau = 1 f* = f_eq.
-        // Lane pairs: (x, y) components, then the directions (1, 2), (3, 4),
-        // (5, 6), (7, 8).
-        const float2 u = div2(fma2(splat(p.tau), F, make_float2(n.jx, n.jy)), splat(-n.rho), splat(rinv));
-        const float om = fmaf(-1.5f, fmaf(u.x, u.x, __fmul_rn(u.y, u.y)), 1.f);
-        const float r9 = div1(n.rho, -9.f, 1.f / 9.f);
-        const float w0r = __fmul_rn(4.f, r9), w2r = __fmul_rn(0.25f, r9);
-        const float2 dg = make_float2(__fadd_rn(u.x, u.y), __fsub_rn(u.y, u.x));  // e5.u, e6.u
-        // f_eq_a = w_a rho (1 + 3 c + 4.5 c^2 - 1.5 u^2) with c = +-(e_a . u):
-        // (-c)(4.5(-c) + 3) = c (4.5 c - 3) exactly
-        const float2 oms = splat(om);
-        auto polyp = [oms](float2 c) { return fma2(c, fma2(splat(4.5f), c, splat(3.f)), oms); };
-        auto polym = [oms](float2 c) { return fma2(c, fma2(splat(4.5f), c, splat(-3.f)), oms); };
         float fs[9];
-        fs[0] = __fmul_rn(w0r, om);
-        const float2 f12 = mul2(splat(r9), polyp(u)), f34 = mul2(splat(r9), polym(u));
-        const float2 f56 = mul2(splat(w2r), polyp(dg)), f78 = mul2(splat(w2r), polym(dg));
-        fs[1] = f12.x; fs[2] = f12.y; fs[3] = f34.x; fs[4] = f34.y;
-        fs[5] = f56.x; fs[6] = f56.y; fs[7] = f78.x; fs[8] = f78.y;
-        if (!T1 && p.tau != 1.f) {
-#pragma unroll
-            for (int a = 0; a < 9; ++a) fs[a] = fmaf(__fsub_rn(fs[a], n.f[a]), p.inv_tau, n.f[a]);
-        }
+        relax_node<T1>(n, F, rinv, p, fs);
         float* o = fout + r * g.pitch + x;
 #pragma unroll
         for (int a = 0; a < 9; ++a) o[a * g.plane] = fs[a];
@@ -746,6 +760,34 @@ __device__ __forceinline__ void pull_dev(const float* __restrict__ s0m, const fl
     n.sb = sb;
 }
 
+// The same in deviation form: q holds the raw deviations d*_a = f*_a - w_a rho
+// (the post-collision density is rho itself).
+template <typename T, bool T1>
+__device__ __forceinline__ void relax_dev(const PulledDev& n, float2 F, float rinv, const Phys& p, float2 (&q)[4])
+{
+    // lane pairs as in relax_node; q[k] holds d*_(2k+1) and d*_(2k+2)
+    const float2 u = div2(fma2(splat(p.tau), F, make_float2(n.jx, n.jy)), splat(-n.rho), splat(rinv));
+    const float nusq = __fmul_rn(-1.5f, fmaf(u.x, u.x, __fmul_rn(u.y, u.y)));
+    // power-of-two scaling to raw units: exact
+    const float w1r = __fmul_rn(div1(n.rho, -9.f, 1.f / 9.f), RawScale<T>::scale);
+    const float w2r = __fmul_rn(0.25f, w1r);
+    const float2 dg = make_float2(__fadd_rn(u.x, u.y), __fsub_rn(u.y, u.x));  // e5.u, e6.u
+    const float2 nus = splat(nusq);
+    auto dpolyp = [nus](float2 c) { return fma2(c, fma2(splat(4.5f), c, splat(3.f)), nus); };
+    auto dpolym = [nus](float2 c) { return fma2(c, fma2(splat(4.5f), c, splat(-3.f)), nus); };
+    q[0] = mul2(splat(w1r), dpolyp(u));
+    q[1] = mul2(splat(w1r), dpolym(u));
+    q[2] = mul2(splat(w2r), dpolyp(dg));
+    q[3] = mul2(splat(w2r), dpolym(dg));
+    if (!T1 && p.tau != 1.f) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const float ga = n.g[2 * k + 1], gb = n.g[2 * k + 2];
+            q[k] = make_float2(fmaf(__fsub_rn(q[k].x, ga), p.inv_tau, ga), fmaf(__fsub_rn(q[k].y, gb), p.inv_tau, gb));
+        }
+    }
+}
+
 // Collision in deviation form: stores rho in plane 0 and the raw
 // d*_a = f*_a - w_a rho after it (the equilibrium's deviation part
 // w_a rho (3 c + 4.5 c^2 - 1.5 u^2) is formed without its leading 1). For
@@ -760,28 +802,8 @@ __device__ __forceinline__ void collide_dev(const PulledDev& n, const float* pm,
     const float2 F = node_force(n, pm, pc, pp, t, p);
     const float rinv = rcp_approx(n.rho);
     if constexpr (MODE == kStep || MODE == kStepObs) {
-        // lane pairs as in collide_node; q[k] holds d*_(2k+1) and d*_(2k+2)
-        const float2 u = div2(fma2(splat(p.tau), F, make_float2(n.jx, n.jy)), splat(-n.rho), splat(rinv));
-        const float nusq = __fmul_rn(-1.5f, fmaf(u.x, u.x, __fmul_rn(u.y, u.y)));
-        // power-of-two scaling to raw units: exact
-        const float w1r = __fmul_rn(div1(n.rho, -9.f, 1.f / 9.f), RawScale<T>::scale);
-        const float w2r = __fmul_rn(0.25f, w1r);
-        const float2 dg = make_float2(__fadd_rn(u.x, u.y), __fsub_rn(u.y, u.x));  // e5.u, e6.u
-        const float2 nus = splat(nusq);
-        auto dpolyp = [nus](float2 c) { return fma2(c, fma2(splat(4.5f), c, splat(3.f)), nus); };
-        auto dpolym = [nus](float2 c) { return fma2(c, fma2(splat(4.5f), c, splat(-3.f)), nus); };
         float2 q[4];
-        q[0] = mul2(splat(w1r), dpolyp(u));
-        q[1] = mul2(splat(w1r), dpolym(u));
-        q[2] = mul2(splat(w2r), dpolyp(dg));
-        q[3] = mul2(splat(w2r), dpolym(dg));
-        if (!T1 && p.tau != 1.f) {
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const float ga = n.g[2 * k + 1], gb = n.g[2 * k + 2];
-                q[k] = make_float2(fmaf(__fsub_rn(q[k].x, ga), p.inv_tau, ga), fmaf(__fsub_rn(q[k].y, gb), p.inv_tau, gb));
-            }
-        }
+        relax_dev<T, T1>(n, F, rinv, p, q);
         const int o = r * g.pitch + x;
         fout0[o] = n.rho;
         if constexpr (sizeof(T) == 2) {
