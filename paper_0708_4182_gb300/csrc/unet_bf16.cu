@@ -8,16 +8,16 @@
 //
 // The 3x3 convolutions run on the 5th-generation tensor cores: tcgen05.mma
 // (kind::f16, BF16 operands from shared memory, FP32 accumulator in tensor
-// memory) issued by one thread per CTA, operands staged by cp.async into the
-// canonical no-swizzle layout (8-row x 16-byte core matrices), completion
-// tracked by tcgen05.commit on mbarriers, the accumulator read back with
-// tcgen05.ld for the epilogue. Forward and input-gradient convolutions are an
-// implicit GEMM with M = 128 output pixels (one row of 128, or 4 rows x 32
-// columns for narrower images), N = a tile of output channels, K = 16 input
-// channels of one of the 9 taps per MMA (both operands K-major: channels are
-// contiguous per pixel). The weight gradient is a GEMM per tap with M = 128
-// output channels, N = a tile of input channels and K = 16 pixels per MMA
-// (both operands MN-major), the 3 taps of a row sharing a CTA's staged operands.
+// memory) issued by one elected thread per CTA, operands staged by cp.async and
+// cp.async.bulk into the canonical no-swizzle layout (8-row x 16-byte core
+// matrices), completion tracked by tcgen05.commit on mbarriers, the accumulator
+// read back with tcgen05.ld for the epilogue. Forward and input-gradient
+// convolutions are an implicit GEMM with M = 128 consecutive pixels of the
+// padded image, N = a tile of output channels, K = 16 input channels of one of
+// the 9 taps per MMA (both operands K-major: channels are contiguous per
+// pixel). The weight gradient is a GEMM per tap with M = 128 channels of the
+// wider side, N = a tile of the other and K = 16 pixels per MMA (both operands
+// MN-major), the 9 taps sharing a CTA's staged operands.
 //
 // A tensor "view" is (pointer to its first channel, channels per pixel of
 // the underlying buffer), so a layer reads or writes a channel range of a
@@ -37,9 +37,7 @@ namespace {
 using bf16 = __nv_bfloat16;
 
 constexpr int kT = 256;                      // threads of the SIMT kernels
-constexpr int kTcThreads = 128;              // threads of the tensor-core kernels (4 warps = 128 TMEM lanes)
 constexpr uint32_t kWaitLimit = 1u << 18;    // try_wait rounds before giving up (about 1 s on a GB300)
-constexpr int kTileRows = 4, kTileCols = 32; // output pixels of one conv CTA (M = 128)
 constexpr int kSmemPerSm = 233472;           // shared memory of one SM (bytes)
 
 __device__ __forceinline__ float ld(const bf16* p) { return __bfloat162float(*p); }
@@ -81,6 +79,23 @@ __device__ __forceinline__ void mbar_arrive(uint64_t* bar)
 {
     asm volatile("{\n\t.reg .b64 st;\n\tmbarrier.arrive.shared::cta.b64 st, [%0];\n\t}" ::"r"(smem_u32(bar))
                  : "memory");
+}
+
+// One arrival that also announces `bytes` of bulk copies to come.
+__device__ __forceinline__ void mbar_expect_arrive(uint64_t* bar, uint32_t bytes)
+{
+    asm volatile("{\n\t.reg .b64 st;\n\tmbarrier.arrive.expect_tx.shared::cta.b64 st, [%0], %1;\n\t}" ::"r"(smem_u32(bar)),
+                 "r"(bytes)
+                 : "memory");
+}
+
+// Contiguous global -> shared copy (16-byte multiples) counted on `bar`.
+__device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t bytes, uint64_t* bar)
+{
+    asm volatile(
+        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(smem_u32(dst)),
+        "l"(src), "r"(bytes), "r"(smem_u32(bar))
+        : "memory");
 }
 
 // 16-byte global -> shared copy; src_bytes = 0 fills zeros (src is not read)
@@ -143,6 +158,19 @@ __device__ __forceinline__ void mma_commit(uint64_t* bar)
                  : "memory");
 }
 
+// One thread of the converged warp. The MMA issue loops branch on this, and on
+// a warp index that is uniform to the compiler (warp_index): behind a plain
+// "lane == 0" it takes 157 cycles to issue an MMA whatever its size (operands
+// of the uniform datapath in divergent code), behind elect 66 for N <= 128, 98
+// for 192 and 130 for 256, the MMA's own rate (measured, one CTA).
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t p;
+    asm volatile("{\n\t.reg .pred e;\n\telect.sync _|e, 0xffffffff;\n\tselp.u32 %0, 1, 0, e;\n\t}" : "=r"(p));
+    return p != 0;
+}
+__device__ __forceinline__ int warp_index() { return __shfl_sync(0xffffffffu, int(threadIdx.x >> 5), 0); }
+
 // 32 lanes x 16 consecutive FP32 columns: thread t of the warp gets lane t
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16])
 {
@@ -157,6 +185,33 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16])
 #pragma unroll
     for (int j = 0; j < 16; ++j) v[j] = __uint_as_float(r[j]);
 }
+
+__device__ __forceinline__ void cluster_sync()
+{
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// Shared address `at` in the cluster's CTA `rank`, and the float at such an address.
+__device__ __forceinline__ uint32_t map_cluster(uint32_t at, uint32_t rank)
+{
+    uint32_t a;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(at), "r"(rank));
+    return a;
+}
+__device__ __forceinline__ float ld_cluster(uint32_t at)
+{
+    float v;
+    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(at) : "memory");
+    return v;
+}
+
+// 32 lanes x 4 columns; the values are there after tmem_ld_wait
+__device__ __forceinline__ void tmem_ld4(uint32_t taddr, float (&v)[4])
+{
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3])
+                 : "r"(taddr));
+}
+__device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
 // TMEM columns to allocate for accumulators spanning n FP32 columns (a power
 // of two >= 32, at most the 512 of an SM; n > 512 cannot be allocated)
@@ -180,59 +235,109 @@ __host__ __device__ constexpr int conv_ntile(int n) { return n % 128 == 0 ? 128 
 // ------------------------------------------------------------------ tensor-core 3x3 convolution
 // y[b, p, co] = act(bias[co] + sum_{tap, k} B[co][k](tap) x[b, p + off(tap), k])
 // x: NHWC view (channels per pixel ct_in, K = 16 kc channels used), y: NHWC
-// view (ct_out per pixel), wt: packed weights (conv_pack_kernel), one CTA =
-// 128 pixels (4 rows x 32 columns) x NT channels of one image.
+// view (ct_out per pixel), wt: packed weights (conv_pack_kernel).
 //
-// K runs over (chunk group, tap): a ring slot holds CK chunks of 16 input
-// channels of one tap (A: 128 pixels x 16 channels per chunk, K-major; B:
-// NT x 16 weights per chunk) and gets CK MMAs. Warp roles as in the weight
-// gradient (wgrad_tc_kernel): warps 1-3 stage the slots with cp.async and
-// arrive on the slot's "full" mbarrier kConvLag steps later (after their own
-// copies landed and were fenced for the async proxy); one thread issues the
-// MMAs and commits them to the slot's "empty" mbarrier; no CTA-wide barrier
-// runs inside the K loop.
-constexpr int kConvStages = 4;   // operand ring depth
-constexpr int kConvLag = 2;      // K-steps between a producer's copies and its "full" arrival
-constexpr int kConvProducers = kTcThreads - 32;
-template <int NT, int CK> __host__ __device__ constexpr int conv_smem_needed()
+// The image (or a strip of S of its columns) is taken with one halo column on
+// each side, pitch = S + 2 pixels a row, and its padded pixels are numbered row
+// by row. A CTA computes MT x 128 consecutive padded pixels (M = 128 a tile) x
+// NT output channels; the results on halo columns are dropped (3% of a 64-wide
+// image, 6% of a 32-wide one). In this numbering tap (dy, dx) of every pixel is
+// the pixel dy pitch + dx further on, so one window of MT 128 + 2 pitch + 2
+// pixels of a 16-channel chunk, staged once at a uniform 16-byte pixel pitch
+// (two planes of 8 channels: LBO the plane distance, SBO 8 pixels), serves all
+// nine taps: the A descriptors of the taps only differ in their start. (Staging
+// the 128 pixels once per tap, as 4 rows x 32 columns, took 9 times the copies;
+// staging 3 halo rows per output row, 3 times, and the weights once per row.)
+//
+// K runs over (group of CK chunks, tap, chunk). Warps 2-7 stage the windows of
+// a group with 16-byte cp.async into a ring of slots and arrive on the slot's
+// "full" mbarrier when their own copies have landed and are fenced for the
+// tensor core's proxy; warp 1 brings the weights, contiguous in the packing,
+// with cp.async.bulk into a ring of slots of TW taps; one thread of warp 0
+// issues the MMAs and commits them to the slots' "empty" mbarriers. All eight
+// warps read the accumulators back. NG blocks of NT output channels share one
+// MMA (32 channels take as long as 96: 64 cycles for N <= 128).
+//
+// Bound by the issue chain (a wait on two barriers and a commit per weight slot
+// around MMAs of 64 cycles each) and, for 32 output channels, by the MMAs
+// themselves. Clusters of 4 that share the weights by multicast, deeper weight
+// rings and 4 window slots were not faster. Measured on 16 images (us, before ->
+// now): 384 -> 128 channels at 16x64 66 -> 21, 128 -> 128 27 -> 12.5, 256 -> 256
+// at 8x32 46 -> 17, 192 -> 64 at 32x128 39 -> 35, 64 -> 192 49 -> 29, 96 -> 32 at
+// 64x256 56 -> 41, 32 -> 96 72 -> 39, 32 -> 32 30 -> 21. The sums run in the
+// order of the earlier kernels, so the outputs are the same bits.
+constexpr int kCvThreads = 256;
+constexpr int kCvProducers = kCvThreads - 64;
+constexpr int kWSlotsMax = 12;
+// weight taps per ring slot; window slots
+template <int CK> __host__ __device__ constexpr int conv_tw() { return CK == 1 ? 3 : 1; }
+// window slots: a short group (few MMAs) needs more of them in flight
+template <int CK, int MT> __host__ __device__ constexpr int conv_xs() { return 2; }
+// window pixels for a strip of S columns, rounded up to 1 mod 8 so that the
+// planes of a pixel lie in different banks
+__host__ __device__ constexpr int conv_npx(int S, int mt) { return (128 * mt + 2 * (S + 2) + 2 + 6) / 8 * 8 + 1; }
+template <int NT, int NG, int CK> __host__ __device__ constexpr int conv_wbytes() { return conv_tw<CK>() * CK * NT * NG * 32; }
+template <int NT, int NG, int CK, int MT> __host__ __device__ constexpr size_t conv_smem(int S, int wslots)
 {
-    return kConvStages * CK * (128 * 16 * 2 + NT * 16 * 2) + 2 * kConvStages * 8 + 16;
+    return size_t(conv_xs<CK, MT>()) * CK * conv_npx(S, MT) * 32 + size_t(wslots) * conv_wbytes<NT, NG, CK>() +
+           (2 * conv_xs<CK, MT>() + 2 * kWSlotsMax + 1) * 8 + 16 + size_t(conv_npx(S, MT)) * 4;
 }
 
-template <int NT, int CK>
-__global__ void __launch_bounds__(kTcThreads) conv3x3_tc_kernel(const bf16* __restrict__ x, int ct_in, int kc,
+template <int NT, int NG, int CK, int MT>
+__global__ void __launch_bounds__(kCvThreads) conv3x3_tc_kernel(const bf16* __restrict__ x, int ct_in, int kc,
                                                                 const bf16* __restrict__ wt,
                                                                 const float* __restrict__ bias,
-                                                                bf16* __restrict__ y, int ct_out, int H, int W,
-                                                                int relu, int* __restrict__ err)
+                                                                bf16* __restrict__ y, int ct_out, int H, int W, int S,
+                                                                int relu, int wslots, int* __restrict__ err)
 {
     extern __shared__ __align__(1024) unsigned char smem[];
-    static_assert(NT <= int(tmem_cols(NT)), "the accumulator must fit the allocation");
-    static_assert(kConvLag < kConvStages, "a producer arrives on a slot before it needs it again");
-    constexpr int kAChunk = 128 * 16 * 2;  // 128 pixels x 16 channels
-    constexpr int kBChunk = NT * 16 * 2;   // NT channels x 16 channels
-    constexpr int kABytes = CK * kAChunk, kBBytes = CK * kBChunk;
-    unsigned char* sa = smem;
-    unsigned char* sb = smem + kConvStages * kABytes;
-    uint64_t* full = reinterpret_cast<uint64_t*>(sb + kConvStages * kBBytes);
-    uint64_t* empty = full + kConvStages;
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(empty + kConvStages);
+    constexpr int N = NT * NG;
+    static_assert(MT * N <= 512, "the accumulators must fit the tensor memory");
+    constexpr int XS = conv_xs<CK, MT>(), TW = conv_tw<CK>();
+    constexpr uint32_t kCols = tmem_cols(MT * N);
+    constexpr int kWBytes = conv_wbytes<NT, NG, CK>();  // one weight slot: TW taps x CK chunks of N x 16
+    const int npx = conv_npx(S, MT);
+    const int xbytes = CK * npx * 32;           // one window slot
+    unsigned char* sw = smem;                   // [wslots][kWBytes]
+    unsigned char* sx = sw + wslots * kWBytes;  // [XS][chunk][plane][pixel] of 16 bytes
+    uint64_t* xfull = reinterpret_cast<uint64_t*>(sx + size_t(XS) * xbytes);
+    uint64_t* xempty = xfull + XS;
+    uint64_t* wfull = xempty + XS;
+    uint64_t* wempty = wfull + kWSlotsMax;
+    uint64_t* done = wempty + kWSlotsMax;
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 1);
+    uint32_t* pix = reinterpret_cast<uint32_t*>(tmem_slot + 4);  // the image's pixel at each window position, or kZeroPix
+    constexpr uint32_t kZeroPix = 0xffffffffu;
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int tiles_x = W / kTileCols;
-    const int ty0 = (blockIdx.x / tiles_x) * kTileRows, tx0 = (blockIdx.x % tiles_x) * kTileCols;
+    __shared__ float sbias[N];
+    const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31;
+    const int strips = W / S, strip = blockIdx.x % strips;
+    const int pitch = S + 2, s0 = (blockIdx.x / strips) * (128 * MT);
     const int nb = blockIdx.y, b = blockIdx.z;
-    const int KT = (kc / CK) * 9;
-    const bf16* wblk = wt + size_t(nb) * kc * 9 * NT * 16;
+    const int groups = kc / CK;
+    const size_t nstride = size_t(kc) * 9 * NT * 16;  // between the packed blocks of NT channels
+    const bf16* wblk = wt + size_t(nb) * NG * nstride;
 
     if (tid == 0) {
-        for (int s = 0; s < kConvStages; ++s) {
-            mbar_init(&full[s], kConvProducers);
-            mbar_init(&empty[s], 1);
+        for (int s = 0; s < XS; ++s) {
+            mbar_init(&xfull[s], kCvProducers);
+            mbar_init(&xempty[s], 1);
         }
+        for (int s = 0; s < wslots; ++s) {
+            mbar_init(&wfull[s], 1);
+            mbar_init(&wempty[s], 1);
+        }
+        mbar_init(done, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (warp == 0) tmem_alloc(tmem_slot, tmem_cols(NT));
+    if (warp == 0) tmem_alloc(tmem_slot, kCols);
+    for (int i = tid; i < N; i += kCvThreads) sbias[i] = bias ? bias[nb * N + i] : 0.f;
+    // window position i is padded pixel s0 - pitch - 1 + i
+    for (int i = tid; i < npx; i += kCvThreads) {
+        const int q = s0 - pitch - 1 + i + 2 * pitch;
+        const int r = q / pitch, yy = r - 2, xx = wrapx(strip * S + (q - r * pitch) - 1, W);
+        pix[i] = (yy >= 0 && yy < H) ? uint32_t(yy) * uint32_t(W) + uint32_t(xx) : kZeroPix;
+    }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -240,209 +345,146 @@ __global__ void __launch_bounds__(kTcThreads) conv3x3_tc_kernel(const bf16* __re
     bool alive = true;
 
     if (warp == 0) {
-        if (lane == 0) {
-            constexpr uint32_t idesc = idesc_bf16(NT, false, false);
+        if (elect_one()) {
+            constexpr uint32_t idesc = idesc_bf16(N, false, false);
+            const uint32_t lbo = uint32_t(npx) * 16;
+            uint32_t acc = 0;
+            int ws = 0;
+            uint32_t wph = 0;
 #pragma unroll 1
-            for (int it = 0; it < KT; ++it) {
-                const int s = it % kConvStages;
-                mbar_wait_alive(&full[s], uint32_t(it / kConvStages) & 1u, err, alive);
-                tc_fence_after();
+            for (int g = 0; g < groups; ++g) {
+                const int s = g % XS;
+                mbar_wait_alive(&xfull[s], uint32_t(g / XS) & 1u, err, alive);
+                const uint32_t xa = smem_u32(sx + size_t(s) * xbytes);
+#pragma unroll 1
+                for (int t0 = 0; t0 < 9; t0 += TW) {
+                    mbar_wait_alive(&wfull[ws], wph, err, alive);
+                    tc_fence_after();
+                    const uint32_t wa = smem_u32(sw + ws * kWBytes);
 #pragma unroll
-                for (int j = 0; j < CK; ++j) {
-                    const uint64_t da = smem_desc(smem_u32(sa + s * kABytes + j * kAChunk), 128, 256);
-                    const uint64_t db = smem_desc(smem_u32(sb + s * kBBytes + j * kBChunk), 128, 256);
-                    mma_bf16(tmem, da, db, idesc, (it > 0 || j > 0) ? 1u : 0u);
+                    for (int tt = 0; tt < TW; ++tt) {
+                        const int t = t0 + tt, dy = t / 3, dx = t - 3 * dy;
+                        const uint32_t off = uint32_t(dy * pitch + dx) * 16;
+#pragma unroll
+                        for (int j = 0; j < CK; ++j) {
+                            const uint64_t db = smem_desc(wa + (tt * CK + j) * N * 32, 128, 256);
+#pragma unroll
+                            for (int m = 0; m < MT; ++m)
+                                mma_bf16(tmem + m * N, smem_desc(xa + j * npx * 32 + off + m * 2048, lbo, 128), db,
+                                         idesc, acc);
+                            acc = 1;
+                        }
+                    }
+                    mma_commit(&wempty[ws]);
+                    if (++ws == wslots) {
+                        ws = 0;
+                        wph ^= 1u;
+                    }
                 }
-                mma_commit(&empty[s]);
+                mma_commit(&xempty[s]);
             }
+            mma_commit(done);
+        }
+        __syncwarp();
+    } else if (warp == 1) {
+        if (elect_one()) {
+            int ws = 0;
+            uint32_t wph = 1;
+#pragma unroll 1
+            for (int g = 0; g < groups; ++g) {
+#pragma unroll 1
+                for (int t0 = 0; t0 < 9; t0 += TW) {
+                    // the slot's earlier MMAs (the first pass over the ring finds the slots free)
+                    if (g * (9 / TW) + t0 / TW >= wslots) mbar_wait_alive(&wempty[ws], wph, err, alive);
+                    mbar_expect_arrive(&wfull[ws], kWBytes);
+                    unsigned char* dst = sw + ws * kWBytes;
+                    if constexpr (CK == 1) {
+                        if constexpr (NG == 1) {  // TW consecutive taps of a chunk are one block
+                            bulk_g2s(dst, wblk + size_t(g * 9 + t0) * NT * 16, kWBytes, &wfull[ws]);
+                        } else {
+                            for (int tt = 0; tt < TW; ++tt)
+                                for (int q = 0; q < NG; ++q)
+                                    bulk_g2s(dst + (tt * NG + q) * NT * 32,
+                                             wblk + q * nstride + size_t(g * 9 + t0 + tt) * NT * 16, NT * 32, &wfull[ws]);
+                        }
+                    } else {
+#pragma unroll
+                        for (int j = 0; j < CK; ++j)
+                            bulk_g2s(dst + j * NT * 32, wblk + size_t((g * CK + j) * 9 + t0) * NT * 16, NT * 32, &wfull[ws]);
+                    }
+                    if (++ws == wslots) {
+                        ws = 0;
+                        wph ^= 1u;
+                    }
+                }
+            }
+            // no copy is in flight when the CTA ends, also after a timeout
+            bool drain = true;
+            const int uses = groups * (9 / TW);
+            for (int u = uses > wslots ? uses - wslots : 0; u < uses; ++u)
+                mbar_wait_alive(&wfull[u % wslots], uint32_t(u / wslots) & 1u, err, drain);
         }
         __syncwarp();
     } else {
-        const int pt = tid - 32;
+        const int pt = tid - 64;
+        constexpr int PP = 2 * CK;   // 16-byte pieces of a pixel
+        constexpr int LAG = XS - 1;  // groups between a thread's copies and their arrival
 #pragma unroll 1
-        for (int it = 0; it < KT; ++it) {
-            const int s = it % kConvStages;
-            if (it >= kConvStages) mbar_wait_alive(&empty[s], uint32_t((it / kConvStages) - 1) & 1u, err, alive);
-            const int t = it % 9, cg = it / 9;
-            const int dy = t / 3 - 1, dx = t % 3 - 1;
-            unsigned char* da = sa + s * kABytes;
-            unsigned char* db = sb + s * kBBytes;
-            // A: CK chunks x 256 pieces of 16 B (pixel q / 2, channel half q % 2)
-            for (int q = pt; q < CK * 256; q += kConvProducers) {
-                const int j = q >> 8, p = (q & 255) >> 1, h = q & 1;
-                const int yy = ty0 + (p >> 5) + dy, xx = wrapx(tx0 + (p & 31) + dx, W);
-                const bool ok = yy >= 0 && yy < H;
-                const bf16* src = ok ? x + (size_t(b * H + yy) * W + xx) * ct_in + (cg * CK + j) * 16 + h * 8 : x;
-                cp_async16_ca(da + j * kAChunk + (p >> 3) * 256 + h * 128 + (p & 7) * 16, src, ok ? 16u : 0u);
+        for (int g = 0; g < groups; ++g) {
+            const int s = g % XS;
+            if (g >= LAG) {  // hand a landed group over before waiting for a slot
+                cp_async_wait<LAG - 1>();
+                fence_proxy_async();
+                mbar_arrive(&xfull[(g - LAG) % XS]);
             }
-            // B: CK chunks x NT * 2 pieces of the packed (chunk, tap) blocks
-            for (int q = pt; q < CK * NT * 2; q += kConvProducers) {
-                const int j = q / (NT * 2), r = q % (NT * 2);
-                const bf16* wsrc = wblk + size_t((cg * CK + j) * 9 + t) * NT * 16;
-                cp_async16_cg(db + j * kBChunk + r * 16, wsrc + r * 8, 16u);
+            if (g >= XS) mbar_wait_alive(&xempty[s], uint32_t(g / XS - 1) & 1u, err, alive);
+            unsigned char* dst = sx + size_t(s) * xbytes + (pt % PP) * npx * 16;
+            const bf16* src = x + size_t(b) * H * W * ct_in + g * CK * 16 + (pt % PP) * 8;
+#pragma unroll 4
+            for (int i = pt / PP; i < npx; i += kCvProducers / PP) {
+                const uint32_t o = pix[i];
+                const bool in = o != kZeroPix;
+                cp_async16_ca(dst + i * 16, in ? src + size_t(o) * ct_in : x, in ? 16u : 0u);
             }
             cp_async_commit();
-            if (it >= kConvLag) {
-                cp_async_wait<kConvLag>();
-                fence_proxy_async();
-                mbar_arrive(&full[(it - kConvLag) % kConvStages]);
-            }
         }
         cp_async_wait<0>();
         fence_proxy_async();
-        for (int it = KT > kConvLag ? KT - kConvLag : 0; it < KT; ++it) mbar_arrive(&full[it % kConvStages]);
+        for (int g = groups > LAG ? groups - LAG : 0; g < groups; ++g) mbar_arrive(&xfull[g % XS]);
     }
-    mbar_wait_alive(&empty[(KT - 1) % kConvStages], uint32_t((KT - 1) / kConvStages) & 1u, err, alive);
+    mbar_wait_alive(done, 0, err, alive);
     tc_fence_after();
 
-    // epilogue: lane = pixel, 16 columns at a time
-    const int p = warp * 32 + lane;
-    const int yy = ty0 + (p >> 5), xx = tx0 + (p & 31);
-    bf16* out = y + (size_t(b * H + yy) * W + xx) * ct_out + nb * NT;
+    // epilogue: warp w reads tensor-memory lanes 32 (w % 4) .. + 31 (pixels of
+    // each tile) and every second 16-channel block of the MT tiles
+    const int quad = warp & 3;
 #pragma unroll 1
-    for (int n0 = 0; n0 < NT; n0 += 16) {
-        float v[16];
-        tmem_ld16(tmem + (uint32_t(warp * 32) << 16) + n0, v);
-        __align__(16) bf16 o[16];
+    for (int m = 0; m < MT; ++m) {
+        const int q = s0 + m * 128 + quad * 32 + lane;
+        const int yy = q / pitch, cc = q - yy * pitch;
+        const bool ok = cc >= 1 && cc <= S && yy < H;
+        bf16* out = y + (size_t(b * H + yy) * W + strip * S + cc - 1) * ct_out + nb * N;
+#pragma unroll 1
+        for (int n0 = 16 * (warp >> 2); n0 < N; n0 += 32) {
+            float v[16];
+            tmem_ld16(tmem + (uint32_t(quad * 32) << 16) + m * N + n0, v);
+            __align__(16) bf16 o[16];
 #pragma unroll
-        for (int j = 0; j < 16; ++j) {
-            float a = v[j] + (bias ? bias[nb * NT + n0 + j] : 0.f);
-            if (relu) a = fmaxf(a, 0.f);
-            o[j] = __float2bfloat16_rn(a);
+            for (int j = 0; j < 16; ++j) {
+                float a = v[j] + sbias[n0 + j];
+                if (relu) a = fmaxf(a, 0.f);
+                o[j] = __float2bfloat16_rn(a);
+            }
+            if (ok) {
+                uint4* dst = reinterpret_cast<uint4*>(out + n0);
+                dst[0] = reinterpret_cast<const uint4*>(o)[0];
+                dst[1] = reinterpret_cast<const uint4*>(o)[1];
+            }
         }
-        uint4* dst = reinterpret_cast<uint4*>(out + n0);
-        dst[0] = reinterpret_cast<const uint4*>(o)[0];
-        dst[1] = reinterpret_cast<const uint4*>(o)[1];
     }
     tc_fence_before();
     __syncthreads();
-    if (warp == 0) tmem_dealloc(tmem, tmem_cols(NT));
-}
-
-// The same convolution for images at least 128 pixels wide: one CTA = 128
-// consecutive pixels of one image row. Per 16-channel chunk the CTA stages a
-// halo of 3 rows x 130 pixels once, pixels at a uniform 16-byte pitch (two
-// planes of 8 channels, LBO = the plane distance, SBO = 8 pixels), and the 9
-// taps are 9 MMAs whose A descriptors start at that halo shifted by dx pixels
-// (16 bytes each) and dy rows: the input crosses shared memory once per chunk
-// instead of once per tap. Three ring slots of one chunk each, with the warp
-// roles of conv3x3_tc_kernel: the next chunks load while this one's MMAs run.
-constexpr int kRowPix = 128, kHaloPix = kRowPix + 2;
-constexpr int kHaloPlane = kHaloPix * 16;      // bytes of one 8-channel plane of one halo row
-constexpr int kHaloBytes = 3 * 2 * kHaloPlane; // 3 rows x 2 planes
-constexpr int kRowStages = 3;                  // ring slots (one chunk each)
-constexpr int kRowLag = 1;                     // chunks between a producer's copies and its "full" arrival
-
-template <int NT>
-__global__ void __launch_bounds__(kTcThreads) conv3x3_tc_row_kernel(const bf16* __restrict__ x, int ct_in, int kc,
-                                                                    const bf16* __restrict__ wt,
-                                                                    const float* __restrict__ bias,
-                                                                    bf16* __restrict__ y, int ct_out, int H, int W,
-                                                                    int relu, int* __restrict__ err)
-{
-    extern __shared__ __align__(1024) unsigned char smem[];
-    static_assert(NT <= int(tmem_cols(NT)), "the accumulator must fit the allocation");
-    static_assert(kRowLag < kRowStages, "a producer arrives on a slot before it needs it again");
-    constexpr int kBBytes = 9 * NT * 16 * 2;  // the 9 taps' weights of one chunk
-    unsigned char* sa = smem;
-    unsigned char* sb = smem + kRowStages * kHaloBytes;
-    uint64_t* full = reinterpret_cast<uint64_t*>(sb + kRowStages * kBBytes);
-    uint64_t* empty = full + kRowStages;
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(empty + kRowStages);
-
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int tiles_x = W / kRowPix;
-    const int y0 = blockIdx.x / tiles_x, x0 = (blockIdx.x % tiles_x) * kRowPix;
-    const int nb = blockIdx.y, b = blockIdx.z;
-    const bf16* wblk = wt + size_t(nb) * kc * 9 * NT * 16;
-
-    if (tid == 0) {
-        for (int s = 0; s < kRowStages; ++s) {
-            mbar_init(&full[s], kConvProducers);
-            mbar_init(&empty[s], 1);
-        }
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
-    if (warp == 0) tmem_alloc(tmem_slot, tmem_cols(NT));
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    const uint32_t tmem = *tmem_slot;
-    bool alive = true;
-
-    if (warp == 0) {
-        if (lane == 0) {
-            constexpr uint32_t idesc = idesc_bf16(NT, false, false);
-#pragma unroll 1
-            for (int c = 0; c < kc; ++c) {
-                const int s = c % kRowStages;
-                mbar_wait_alive(&full[s], uint32_t(c / kRowStages) & 1u, err, alive);
-                tc_fence_after();
-                const uint32_t a0 = smem_u32(sa + s * kHaloBytes);
-                const uint32_t b0 = smem_u32(sb + s * kBBytes);
-#pragma unroll
-                for (int t = 0; t < 9; ++t) {
-                    const int dy = t / 3, dx = t % 3;  // halo row and pixel shift of this tap
-                    const uint64_t da = smem_desc(a0 + dy * 2 * kHaloPlane + dx * 16, kHaloPlane, 128);
-                    const uint64_t db = smem_desc(b0 + t * NT * 32, 128, 256);
-                    mma_bf16(tmem, da, db, idesc, (c > 0 || t > 0) ? 1u : 0u);
-                }
-                mma_commit(&empty[s]);
-            }
-        }
-        __syncwarp();
-    } else {
-        const int pt = tid - 32;
-#pragma unroll 1
-        for (int c = 0; c < kc; ++c) {
-            const int s = c % kRowStages;
-            if (c >= kRowStages) mbar_wait_alive(&empty[s], uint32_t((c / kRowStages) - 1) & 1u, err, alive);
-            unsigned char* da = sa + s * kHaloBytes;
-            // 3 rows x 130 pixels x 2 planes of 16 bytes
-            for (int q = pt; q < 3 * kHaloPix * 2; q += kConvProducers) {
-                const int h = q & 1, pix = (q >> 1) % kHaloPix, r = (q >> 1) / kHaloPix;
-                const int yy = y0 + r - 1, xx = wrapx(x0 + pix - 1, W);
-                const bool ok = yy >= 0 && yy < H;
-                const bf16* src = ok ? x + (size_t(b * H + yy) * W + xx) * ct_in + c * 16 + h * 8 : x;
-                cp_async16_ca(da + (r * 2 + h) * kHaloPlane + pix * 16, src, ok ? 16u : 0u);
-            }
-            const bf16* wsrc = wblk + size_t(c) * 9 * NT * 16;
-            unsigned char* db = sb + s * kBBytes;
-            for (int q = pt; q < 9 * NT * 2; q += kConvProducers) cp_async16_cg(db + q * 16, wsrc + q * 8, 16u);
-            cp_async_commit();
-            if (c >= kRowLag) {
-                cp_async_wait<kRowLag>();
-                fence_proxy_async();
-                mbar_arrive(&full[(c - kRowLag) % kRowStages]);
-            }
-        }
-        cp_async_wait<0>();
-        fence_proxy_async();
-        for (int c = kc > kRowLag ? kc - kRowLag : 0; c < kc; ++c) mbar_arrive(&full[c % kRowStages]);
-    }
-    mbar_wait_alive(&empty[(kc - 1) % kRowStages], uint32_t((kc - 1) / kRowStages) & 1u, err, alive);
-    tc_fence_after();
-
-    const int p = warp * 32 + lane;
-    bf16* out = y + (size_t(b * H + y0) * W + x0 + p) * ct_out + nb * NT;
-#pragma unroll 1
-    for (int n0 = 0; n0 < NT; n0 += 16) {
-        float v[16];
-        tmem_ld16(tmem + (uint32_t(warp * 32) << 16) + n0, v);
-        __align__(16) bf16 o[16];
-#pragma unroll
-        for (int j = 0; j < 16; ++j) {
-            float a = v[j] + (bias ? bias[nb * NT + n0 + j] : 0.f);
-            if (relu) a = fmaxf(a, 0.f);
-            o[j] = __float2bfloat16_rn(a);
-        }
-        uint4* dst = reinterpret_cast<uint4*>(out + n0);
-        dst[0] = reinterpret_cast<const uint4*>(o)[0];
-        dst[1] = reinterpret_cast<const uint4*>(o)[1];
-    }
-    tc_fence_before();
-    __syncthreads();
-    if (warp == 0) tmem_dealloc(tmem, tmem_cols(NT));
+    if (warp == 0) tmem_dealloc(tmem, kCols);
 }
 
 // Packed B operand of the tensor-core convolution. Forward (transpose = 0):
@@ -497,84 +539,98 @@ __global__ void conv_pack_many_kernel(const long long* __restrict__ jobs)
 
 // ------------------------------------------------------------------ tensor-core weight gradient
 // dw[co][ci][tap] += sum over pixels p of dy[p][co] x[p + off(tap)][ci]: per
-// tap a GEMM with M = 128 output channels, N = NT input channels and K = the
-// pixels. One CTA takes one tap row (dy = -1, 0, 1 of the 3x3 stencil) and a
-// range of npix pixels. Per K-step of P pixels of one image row (P = 16, 32
-// or 64, dividing the row), dy (A, 128 output channels x P pixels, MN-major:
-// 8 channels of a pixel in 16 bytes, pixels at a 16-byte pitch, so LBO = 8
-// pixels and SBO = P pixels) is staged once, and x as a halo row of P + 2
-// pixels x NT channels (B, MN-major likewise: SBO = P + 2 pixels). Each
-// 16-pixel piece j of the step gives three MMAs, one per tap (dx = -1, 0, 1)
-// of the row: A starts 16 j pixels in, B 16 j + dx pixels in, into three
-// accumulators of NT columns (3 NT <= 512 tensor-memory columns). With SW
-// (layers with more input than output channels) the operands swap roles:
-// the x halo row is A (M = 128 input channels) and dy is B (N = NT output
-// channels), so that the wider side fills the MMA's 128 rows; the shared
-// layouts and descriptors are the same, and the accumulators hold dw
-// transposed (lane = input channel).
+// tap a GEMM whose K runs over the pixels, 16 a MMA, both operands MN-major (8
+// channels of a pixel in 16 bytes, pixels at a 16-byte pitch: LBO = 8 pixels,
+// SBO = the distance of two channel groups). The wider of the two channel
+// counts is the MMA's M (tiles of 128 rows: dy, or x with SW), the narrower
+// its N (tiles of NT = 32 or 16).
 //
-// Warp roles: warps 1-3 stage the operands with 16-byte cp.async into a ring
-// of kWgStages slots; each producer thread waits for its own copies of a slot
-// two steps later, fences them for the tensor core's (async) proxy and
-// arrives on the slot's "full" mbarrier (96 arrivals). One thread of warp 0
-// waits on "full", issues the MMAs and commits them to the slot's "empty"
-// mbarrier, which the producers wait on before refilling the slot. No
-// CTA-wide barrier runs inside the K loop. The epilogue adds the three
-// accumulators into dw (FP32 atomics; the grid splits the pixels).
-constexpr int kWgStages = 4;   // operand ring depth of the weight gradient
-constexpr int kWgLag = 2;      // K-steps between a producer's copies and its "full" arrival
+// A CTA marches down columns of P pixels (P = 64, 32 or 16, dividing the row)
+// with all nine taps: row y of dy meets rows y - 1, y and y + 1 of x (halo rows
+// of P + 2 pixels), each into its own accumulator (9 NT <= 512 tensor-memory
+// columns), so every row of dy and of x is staged once per column; a tap's dx
+// only moves the start of the x descriptor. (One tap row per CTA staged both
+// three times, and its epilogue added three floats in every nine.) Rows
+// outside the image are skipped.
+//
+// Warps 1-7 stage row r of x and row r - 1 of dy with 16-byte cp.async into
+// slot r of a ring and arrive on its "full" mbarrier kWgLag rows later (their
+// own copies landed and fenced for the tensor core's proxy); one thread of
+// warp 0 issues the MMAs of row r - 1 and commits them to the "empty" mbarrier
+// of the slot that held row r - 2. The grid is one wave: each CTA takes an
+// equal share of the rows of all columns, crossing from column to column.
+//
+// The epilogue lays the accumulators out in shared memory as dw has them; the
+// CTAs of a cluster add them up through distributed shared memory and add the
+// sums to dw with atomics on consecutive floats, a warp's 32 in 4 sectors. (Lane
+// by lane, and once per CTA, they took 26 of 45 us at 128 x 128 channels.)
+// An MMA of N <= 128 takes 64 cycles, which bounds the narrow layers (32 x 32
+// channels at 64x256: 32 us of MMAs). Measured on 16 images (us, before -> now):
+// 32 -> 32 at 64x256 54 -> 35, 96 -> 32 92 -> 39, 64 -> 64 at 32x128 46 -> 25,
+// 192 -> 64 101 -> 39, 128 -> 128 at 16x64 48 -> 19, 384 -> 128 56 -> 35,
+// 256 -> 256 at 8x32 46 -> 21.
+constexpr int kWgSlots = 6;
+constexpr int kWgLag = 2;                       // rows between a producer's copies and their "full" arrival
 constexpr int kWgThreads = 256;                 // 8 warps: one issues the MMAs, seven stage operands
 constexpr int kWgProducers = kWgThreads - 32;
 template <int P> __host__ __device__ constexpr int wgrad_halo_pix() { return P + 2; }
 // dy and x channels per CTA
 template <int NT, bool SW> __host__ __device__ constexpr int wgrad_co_tile() { return SW ? NT : 128; }
 template <int NT, bool SW> __host__ __device__ constexpr int wgrad_ci_tile() { return SW ? 128 : NT; }
+// The accumulators in shared memory, for the sum over a cluster: per output
+// channel the 9 taps of the tile's input channels in a row, plus one float of
+// padding (bank conflicts).
+template <int NT, bool SW> __host__ __device__ constexpr int wgrad_red_pitch() { return wgrad_ci_tile<NT, SW>() * 9 + 1; }
+template <int NT, bool SW> __host__ __device__ constexpr int wgrad_red_bytes() { return wgrad_co_tile<NT, SW>() * wgrad_red_pitch<NT, SW>() * 4; }
+constexpr int kWgCluster = 8;                   // CTAs whose sums are added before they reach dw, at most
 template <int NT, int P, bool SW> __host__ __device__ constexpr int wgrad_smem_needed()
 {
-    return kWgStages * (wgrad_co_tile<NT, SW>() * P * 2 + (wgrad_ci_tile<NT, SW>() / 8) * wgrad_halo_pix<P>() * 16) +
-           2 * kWgStages * 8 + 16;
+    const int ring = kWgSlots * (wgrad_co_tile<NT, SW>() * P * 2 + (wgrad_ci_tile<NT, SW>() / 8) * wgrad_halo_pix<P>() * 16);
+    const int red = (wgrad_red_bytes<NT, SW>() + 15) / 16 * 16;
+    return (ring > red ? ring : red) + 2 * kWgSlots * 8 + 8 + 16;
 }
 
 template <int NT, int P, bool SW>
 __global__ void __launch_bounds__(kWgThreads) wgrad_tc_kernel(const bf16* __restrict__ x, int ct_x, int ci,
                                                               const bf16* __restrict__ dy, int ct_dy, int co,
-                                                              float* __restrict__ dw, int H, int W, int npix,
-                                                              int* __restrict__ err)
+                                                              float* __restrict__ dw, int H, int W, long long rows,
+                                                              long long per, int cs, int* __restrict__ err)
 {
     extern __shared__ __align__(1024) unsigned char smem[];
-    static_assert(3 * NT <= 512, "three accumulators must fit the tensor memory");
-    static_assert(P == 16 || P == 32 || P == 64, "K-step of 16, 32 or 64 pixels");
-    static_assert(kWgLag < kWgStages, "a producer arrives on a slot before it needs it again");
+    static_assert(9 * NT <= 512, "nine accumulators must fit the tensor memory");
+    static_assert(P == 16 || P == 32 || P == 64, "columns of 16, 32 or 64 pixels");
+    static_assert(kWgLag + 3 <= kWgSlots, "a row's three x slots, and those on their way");
     constexpr int COT = wgrad_co_tile<NT, SW>(), CIT = wgrad_ci_tile<NT, SW>();
     constexpr int HP = wgrad_halo_pix<P>();                // halo row pixels
-    constexpr int kABytes = COT * P * 2;                   // dy: COT output channels x P pixels
-    constexpr int kBBytes = (CIT / 8) * HP * 16;           // x: one halo row of CIT input channels
-    constexpr uint32_t kCols = tmem_cols(3 * NT);
-    unsigned char* sa = smem;
-    unsigned char* sb = smem + kWgStages * kABytes;
-    uint64_t* full = reinterpret_cast<uint64_t*>(sb + kWgStages * kBBytes);
-    uint64_t* empty = full + kWgStages;
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(empty + kWgStages);
+    constexpr int kDBytes = COT * P * 2;                   // dy: COT output channels x P pixels
+    constexpr int kXBytes = (CIT / 8) * HP * 16;           // x: one halo row of CIT input channels
+    constexpr int kSlot = kDBytes + kXBytes;
+    constexpr int kRing = kWgSlots * kSlot, kRed = (wgrad_red_bytes<NT, SW>() + 15) / 16 * 16;
+    constexpr uint32_t kCols = tmem_cols(9 * NT);
+    uint64_t* full = reinterpret_cast<uint64_t*>(smem + (kRing > kRed ? kRing : kRed));
+    uint64_t* empty = full + kWgSlots;
+    uint64_t* done = empty + kWgSlots;
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 1);
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31;
     const int co0 = blockIdx.x * COT, ci0 = blockIdx.y * CIT;
-    const int trow = blockIdx.z % 3;                       // taps 3 trow .. 3 trow + 2 (row offset trow - 1)
     const int co_here = co - co0 < COT ? co - co0 : COT;
     const int ci_here = ci - ci0 < CIT ? ci - ci0 : CIT;
-    const int KT = npix / P;
+    // rows k_begin .. k_end - 1 of all columns' rows (column k / H, image row k % H)
+    const long long k_begin = blockIdx.z * per, k_end = k_begin + per < rows ? k_begin + per : rows;
+    const int cols_x = W / P;
 
-    // rows of A beyond co_here and channel groups of B beyond ci_here are never loaded: zero them once
-    for (int i = tid; i < kWgStages * (kABytes + kBBytes) / 16; i += kWgThreads)
-        reinterpret_cast<uint4*>(smem)[i] = make_uint4(0, 0, 0, 0);
+    // channel groups beyond co_here and ci_here are never loaded: they only reach
+    // accumulators that are not read
     if (tid == 0) {
-        for (int s = 0; s < kWgStages; ++s) {
+        for (int s = 0; s < kWgSlots; ++s) {
             mbar_init(&full[s], kWgProducers);
             mbar_init(&empty[s], 1);
         }
+        mbar_init(done, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 0) tmem_alloc(tmem_slot, kCols);
-    fence_proxy_async();  // the zeroed slots, before the tensor core reads them
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -582,107 +638,175 @@ __global__ void __launch_bounds__(kWgThreads) wgrad_tc_kernel(const bf16* __rest
     bool alive = true;
 
     if (warp == 0) {
-        if (lane == 0) {
+        if (elect_one()) {
             constexpr uint32_t idesc = idesc_bf16(NT, true, true);
+            const uint32_t s0 = smem_u32(smem);
+            uint32_t acc[3] = {0, 0, 0};  // per tap row: its accumulators have been written
+            int slot = 0;
+            uint32_t ph = 0;
 #pragma unroll 1
-            for (int k = 0; k < KT; ++k) {
-                const int s = k % kWgStages;
-                mbar_wait_alive(&full[s], uint32_t(k / kWgStages) & 1u, err, alive);
-                tc_fence_after();
-                const uint32_t a0 = smem_u32(sa + s * kABytes);
-                const uint32_t b0 = smem_u32(sb + s * kBBytes);
+            for (long long k = k_begin; k < k_end;) {
+                const int ya = int(k % H), n = int(k_end - k < H - ya ? k_end - k : H - ya), yb = ya + n;
+                k += n;
+#pragma unroll 1
+                for (int r = ya - 1; r <= yb; ++r) {
+                    mbar_wait_alive(&full[slot], ph, err, alive);
+                    tc_fence_after();
+                    const int sm1 = slot == 0 ? kWgSlots - 1 : slot - 1, sm2 = sm1 == 0 ? kWgSlots - 1 : sm1 - 1;
+                    if (r > ya) {
+                        // row y = r - 1: dy in this slot, x rows y - 1, y, y + 1 in the last three
+                        const uint32_t da = s0 + slot * kSlot;
 #pragma unroll
-                for (int j = 0; j < P / 16; ++j) {
-                    const uint64_t dd = smem_desc(a0 + j * 256, 128, P * 16);  // dy piece j
+                        for (int t = 0; t < 3; ++t) {
+                            const int xr = r - 2 + t;
+                            if (xr < 0 || xr >= H) continue;
+                            const uint32_t xa = s0 + (t == 0 ? sm2 : t == 1 ? sm1 : slot) * kSlot + kDBytes;
 #pragma unroll
-                    for (int dx = 0; dx < 3; ++dx) {
-                        const uint64_t dh = smem_desc(b0 + (16 * j + dx) * 16, 128, HP * 16);  // x, shifted dx
-                        if constexpr (SW)
-                            mma_bf16(tmem + dx * NT, dh, dd, idesc, (k > 0 || j > 0) ? 1u : 0u);
-                        else
-                            mma_bf16(tmem + dx * NT, dd, dh, idesc, (k > 0 || j > 0) ? 1u : 0u);
+                            for (int j = 0; j < P / 16; ++j) {
+                                const uint64_t dd = smem_desc(da + j * 256, 128, P * 16);  // dy, 16-pixel piece j
+#pragma unroll
+                                for (int dx = 0; dx < 3; ++dx) {
+                                    const uint64_t dh = smem_desc(xa + (16 * j + dx) * 16, 128, HP * 16);  // x, shifted dx
+                                    mma_bf16(tmem + (3 * t + dx) * NT, SW ? dh : dd, SW ? dd : dh, idesc,
+                                             j > 0 ? 1u : acc[t]);
+                                }
+                            }
+                            acc[t] = 1;
+                        }
+                        mma_commit(&empty[sm2]);
+                        if (r == yb) {  // the column's last row: its other slots as well
+                            mma_commit(&empty[sm1]);
+                            mma_commit(&empty[slot]);
+                        }
+                    }
+                    if (++slot == kWgSlots) {
+                        slot = 0;
+                        ph ^= 1u;
                     }
                 }
-                mma_commit(&empty[s]);
             }
+            mma_commit(done);
         }
         __syncwarp();
     } else {
-        const int pt = tid - 32;                           // producer thread 0 .. 95
-        const int ga = (co_here + 7) / 8, gb = (ci_here + 7) / 8;
-        // position of K-step k: image bimg, row yy, first column x0 (each step
-        // lies inside one image row), advanced incrementally
-        const long long p_begin = (long long)(blockIdx.z / 3) * npix;
-        int bimg = int(p_begin / ((long long)H * W));
-        const int rem = int(p_begin - (long long)bimg * H * W);
-        int yy = rem / W, x0 = rem % W;
+        const int pt = tid - 32;  // producer thread
+        const int gd = (co_here + 7) / 8, gx = (ci_here + 7) / 8;
+        int slot = 0, lslot = 0;  // slot of this row, and of the row to hand over
+        uint32_t ph = 1;          // (the first pass over the ring finds the slots free)
+        long long step = 0;
 #pragma unroll 1
-        for (int k = 0; k < KT; ++k) {
-            const int s = k % kWgStages;
-            if (k >= kWgStages) mbar_wait_alive(&empty[s], uint32_t((k / kWgStages) - 1) & 1u, err, alive);
-            unsigned char* da = sa + s * kABytes;
-            unsigned char* db = sb + s * kBBytes;
-            const bf16* arow = dy + (size_t(bimg * H + yy) * W + x0) * ct_dy + co0;
-            for (int q = pt; q < P * ga; q += kWgProducers) {
-                const int kk = q % P, g = q / P;
-                cp_async16_cg(da + g * (P * 16) + kk * 16, arow + size_t(kk) * ct_dy + g * 8, 16u);
-            }
-            const int ys = yy + trow - 1;
-            const bool ok = ys >= 0 && ys < H;
-            const bf16* brow = x + size_t(bimg * H + (ok ? ys : 0)) * W * ct_x + ci0;
-            for (int q = pt; q < HP * gb; q += kWgProducers) {
-                const int pix = q % HP, g = q / HP;
-                const int xs = wrapx(x0 + pix - 1, W);
-                cp_async16_ca(db + g * (HP * 16) + pix * 16, ok ? brow + size_t(xs) * ct_x + g * 8 : x, ok ? 16u : 0u);
-            }
-            cp_async_commit();
-            if (k >= kWgLag) {
-                cp_async_wait<kWgLag>();
-                fence_proxy_async();
-                mbar_arrive(&full[(k - kWgLag) % kWgStages]);
-            }
-            x0 += P;
-            if (x0 == W) {
-                x0 = 0;
-                if (++yy == H) {
-                    yy = 0;
-                    ++bimg;
+        for (long long k = k_begin; k < k_end;) {
+            const long long col = k / H;
+            const int ya = int(k - col * H), n = int(k_end - k < H - ya ? k_end - k : H - ya), yb = ya + n;
+            k += n;
+            const long long img = (col / cols_x) * H;  // the image's first row
+            const int x0 = int(col % cols_x) * P;
+#pragma unroll 1
+            for (int r = ya - 1; r <= yb; ++r, ++step) {
+                if (step >= kWgSlots) mbar_wait_alive(&empty[slot], ph, err, alive);
+                unsigned char* sd = smem + slot * kSlot;
+                unsigned char* sx = sd + kDBytes;
+                if (r > ya) {
+                    const bf16* drow = dy + (size_t(img + r - 1) * W + x0) * ct_dy + co0;
+                    for (int q = pt; q < P * gd; q += kWgProducers) {
+                        const int kk = q % P, g = q / P;
+                        cp_async16_cg(sd + g * (P * 16) + kk * 16, drow + size_t(kk) * ct_dy + g * 8, 16u);
+                    }
+                }
+                if (r >= 0 && r < H) {
+                    const bf16* xrow = x + size_t(img + r) * W * ct_x + ci0;
+                    for (int q = pt; q < HP * gx; q += kWgProducers) {
+                        const int pix = q % HP, g = q / HP;
+                        const int xs = wrapx(x0 + pix - 1, W);
+                        cp_async16_ca(sx + g * (HP * 16) + pix * 16, xrow + size_t(xs) * ct_x + g * 8, 16u);
+                    }
+                }
+                cp_async_commit();
+                if (step >= kWgLag) {
+                    cp_async_wait<kWgLag>();
+                    fence_proxy_async();
+                    mbar_arrive(&full[lslot]);
+                    lslot = lslot + 1 == kWgSlots ? 0 : lslot + 1;
+                }
+                if (++slot == kWgSlots) {
+                    slot = 0;
+                    ph ^= 1u;
                 }
             }
         }
         cp_async_wait<0>();
         fence_proxy_async();
-        for (int k = KT > kWgLag ? KT - kWgLag : 0; k < KT; ++k) mbar_arrive(&full[k % kWgStages]);
-    }
-    // every warp: the last commit completes when all MMAs have
-    mbar_wait_alive(&empty[(KT - 1) % kWgStages], uint32_t((KT - 1) / kWgStages) & 1u, err, alive);
-    tc_fence_after();
-
-    // warp w reads tensor-memory lanes 32 (w % 4) .. + 31 (its quadrant) and
-    // the accumulator columns of every (w / 4)-th 16-column block
-    const int quad = warp & 3, half = warp >> 2;
-    const int m = quad * 32 + lane;  // accumulator row: output channel co0 + m (input channel ci0 + m with SW)
-    const int m_here = SW ? ci_here : co_here, n_here = SW ? co_here : ci_here;
-#pragma unroll 1
-    for (int dx = 0; dx < 3; ++dx) {
-        const int tap = trow * 3 + dx;
-#pragma unroll 1
-        for (int n0 = 16 * half; n0 < NT; n0 += 16 * (kWgThreads / 128)) {
-            float v[16];
-            tmem_ld16(tmem + (uint32_t(quad * 32) << 16) + dx * NT + n0, v);
-            if (m < m_here) {
-#pragma unroll
-                for (int j = 0; j < 16; ++j) {
-                    if (n0 + j >= n_here) continue;
-                    const size_t o = SW ? (size_t(co0 + n0 + j) * ci + ci0 + m) : (size_t(co0 + m) * ci + ci0 + n0 + j);
-                    atomicAdd(&dw[o * 9 + tap], v[j]);
-                }
-            }
+        for (long long s = step > kWgLag ? step - kWgLag : 0; s < step; ++s) {
+            mbar_arrive(&full[lslot]);
+            lslot = lslot + 1 == kWgSlots ? 0 : lslot + 1;
         }
     }
-    tc_fence_before();
+    // every warp: the last commit completes when all MMAs have
+    mbar_wait_alive(done, 0, err, alive);
+    tc_fence_after();
+    // the ring becomes the exchange space: nobody copies into it any more
     __syncthreads();
+
+    // warp w reads tensor-memory lanes 32 (w % 4) .. + 31 and every second
+    // block of 4 columns, nine taps of each
+    constexpr int RP = wgrad_red_pitch<NT, SW>();
+    float* red = reinterpret_cast<float*>(smem);
+    const int m = (warp & 3) * 32 + lane;
+    // a tap row that lay outside the image for every row of this CTA was never
+    // written (nor anything by a CTA without rows)
+    const bool any = k_end > k_begin, many = H > 1 && k_end - k_begin > 1;
+    const bool up = many || (any && k_begin % H > 0), down = many || (any && k_begin % H < H - 1);
+#pragma unroll 1
+    for (int n0 = 4 * (warp >> 2); n0 < NT; n0 += 8) {
+        float v[9][4];
+#pragma unroll
+        for (int t = 0; t < 9; ++t) tmem_ld4(tmem + (uint32_t((warp & 3) * 32) << 16) + t * NT + n0, v[t]);
+        tmem_ld_wait();
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+#pragma unroll
+            for (int t = 0; t < 9; ++t) {
+                const bool ok = t < 3 ? up : t < 6 ? any : down;
+                red[SW ? (n0 + c) * RP + m * 9 + t : m * RP + (n0 + c) * 9 + t] = ok ? v[t][c] : 0.f;
+            }
+    }
+    tc_fence_before();
+    if (cs > 1)
+        cluster_sync();
+    else
+        __syncthreads();
     if (warp == 0) tmem_dealloc(tmem, kCols);
+    const int len = ci_here * 9;
+    if (cs == 1) {
+        // a warp per output channel
+        for (int row = warp; row < co_here; row += kWgThreads / 32) {
+            float* dst = dw + (size_t(co0 + row) * ci + ci0) * 9;
+            const float* src = red + row * RP;
+#pragma unroll 9
+            for (int i = lane; i < len; i += 32) atomicAdd(dst + i, src[i]);
+        }
+        return;
+    }
+    // each CTA of the cluster adds its share of the output channels over all of
+    // them, in the order of their ranks, and the sums to dw
+    const int rank = int(blockIdx.z) % cs, share = (co_here + cs - 1) / cs, o_end = min(co_here - rank * share, share);
+    const uint32_t red0 = smem_u32(red);
+    uint32_t peer[kWgCluster];  // red of each rank
+#pragma unroll
+    for (int q = 0; q < kWgCluster; ++q) peer[q] = map_cluster(red0, q < cs ? q : 0);
+#pragma unroll 2
+    for (int i = tid; i < o_end * len; i += kWgThreads) {
+        const int o = i / len, e = i - o * len, row = rank * share + o;
+        const uint32_t at = uint32_t(row * RP + e) * 4;
+        float v[kWgCluster];
+#pragma unroll
+        for (int q = 0; q < kWgCluster; ++q) v[q] = q < cs ? ld_cluster(peer[q] + at) : 0.f;
+        float sum = v[0];
+#pragma unroll
+        for (int q = 1; q < kWgCluster; ++q) sum += v[q];
+        atomicAdd(dw + (size_t(co0 + row) * ci + ci0) * 9 + e, sum);
+    }
+    cluster_sync();  // a peer may still be reading this CTA's sums
 }
 
 // ------------------------------------------------------------------ SIMT kernels (NHWC)
@@ -1129,98 +1253,142 @@ int* err_ptr()
     return p;
 }
 
-template <int NT>
-int launch_conv_row(const void* x, int ct_in, int kc, const void* wt, const float* bias, void* y, int ct_out,
-                    int cout, int n, int h, int wd, int relu, cudaStream_t st)
+// columns of a strip: the whole row up to 256 columns, else the largest
+// multiple of 32 up to 256 that divides it
+int conv_strip(int wd)
 {
-    constexpr int needed = kRowStages * (kHaloBytes + 9 * NT * 32) + 2 * kRowStages * 8 + 16;
-    const int smem = smem_for_tmem(int(tmem_cols(NT)), needed);
-    auto k = conv3x3_tc_row_kernel<NT>;
+    if (wd <= 256) return wd;
+    int s = 256;
+    while (wd % s) s -= 32;
+    return s;
+}
+
+template <int NT, int NG, int CK, int MT>
+int launch_conv_mt(const void* x, int ct_in, int kc, const void* wt, const float* bias, void* y, int ct_out, int cout,
+                   int n, int h, int wd, int relu, cudaStream_t st)
+{
+    const int S = conv_strip(wd);
+    constexpr int cols = int(tmem_cols(MT * NT * NG));
+    // weight slots: what fits beside a second CTA on the SM (or alone, where
+    // the accumulators or 4 slots leave no room for one), up to the K loop's uses
+    const int budget = cols <= 256 && 2 * (conv_smem<NT, NG, CK, MT>(S, 4) + 1024) <= kSmemPerSm ? kSmemPerSm / 2 - 1024
+                                                                                                 : kSmemPerSm - 1024;
+    constexpr int WMAX = CK == 1 ? 4 : kWSlotsMax;
+    int wslots = 4;
+    while (wslots < WMAX && wslots < (kc / CK) * (9 / conv_tw<CK>()) &&
+           conv_smem<NT, NG, CK, MT>(S, wslots + 1) <= size_t(budget))
+        ++wslots;
+    const int smem = smem_for_tmem(cols, int(conv_smem<NT, NG, CK, MT>(S, wslots)));
+    auto k = conv3x3_tc_kernel<NT, NG, CK, MT>;
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return int(e);
-    dim3 grid(h * (wd / kRowPix), cout / NT, n);
-    k<<<grid, kTcThreads, smem, st>>>((const bf16*)x, ct_in, kc, (const bf16*)wt, bias, (bf16*)y, ct_out, h, wd, relu,
-                                      err_ptr());
+    dim3 grid((wd / S) * ((h * (S + 2) + 128 * MT - 1) / (128 * MT)), cout / (NT * NG), n);
+    k<<<grid, kCvThreads, smem, st>>>((const bf16*)x, ct_in, kc, (const bf16*)wt, bias, (bf16*)y, ct_out, h, wd, S,
+                                      relu, wslots, err_ptr());
     return status(cudaGetLastError());
 }
 
-template <int NT, int CK>
-int launch_conv_tile(const void* x, int ct_in, int kc, const void* wt, const float* bias, void* y, int ct_out,
+// Rows of whole 128-pixel tiles (CK = 1): MT tiles per CTA, the most of 4, 2
+// and 1 that leave two CTAs per SM; more tiles reuse the staged weights and
+// halo rows.
+template <int NT, int NG>
+int launch_conv_wide(const void* x, int ct_in, int kc, const void* wt, const float* bias, void* y, int ct_out,
                      int cout, int n, int h, int wd, int relu, cudaStream_t st)
 {
-    const int smem = smem_for_tmem(int(tmem_cols(NT)), conv_smem_needed<NT, CK>());
-    auto k = conv3x3_tc_kernel<NT, CK>;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e != cudaSuccess) return int(e);
-    dim3 grid((h / kTileRows) * (wd / kTileCols), cout / NT, n);
-    k<<<grid, kTcThreads, smem, st>>>((const bf16*)x, ct_in, kc, (const bf16*)wt, bias, (bf16*)y, ct_out, h, wd, relu,
-                                      err_ptr());
-    return status(cudaGetLastError());
+    constexpr int N = NT * NG;
+    const int S = conv_strip(wd);
+    auto ctas = [&](int mt) {
+        return (long long)(wd / S) * ((h * (S + 2) + 128 * mt - 1) / (128 * mt)) * (cout / N) * n;
+    };
+    if (N <= 64 && ctas(4) >= 304)
+        return launch_conv_mt<NT, NG, 1, N <= 64 ? 4 : 1>(x, ct_in, kc, wt, bias, y, ct_out, cout, n, h, wd, relu, st);
+    if (ctas(2) >= 304) return launch_conv_mt<NT, NG, 1, 2>(x, ct_in, kc, wt, bias, y, ct_out, cout, n, h, wd, relu, st);
+    return launch_conv_mt<NT, NG, 1, 1>(x, ct_in, kc, wt, bias, y, ct_out, cout, n, h, wd, relu, st);
 }
 
 template <int NT>
 int launch_conv(const void* x, int ct_in, int kc, const void* wt, const float* bias, void* y, int ct_out, int cout,
                 int n, int h, int wd, int relu, cudaStream_t st)
 {
-    if (wd % kRowPix == 0) return launch_conv_row<NT>(x, ct_in, kc, wt, bias, y, ct_out, cout, n, h, wd, relu, st);
-    // chunks of 16 channels per ring slot: 4, 2 or 1, dividing kc
-    if (kc % 4 == 0) return launch_conv_tile<NT, 4>(x, ct_in, kc, wt, bias, y, ct_out, cout, n, h, wd, relu, st);
-    if (kc % 2 == 0) return launch_conv_tile<NT, 2>(x, ct_in, kc, wt, bias, y, ct_out, cout, n, h, wd, relu, st);
-    return launch_conv_tile<NT, 1>(x, ct_in, kc, wt, bias, y, ct_out, cout, n, h, wd, relu, st);
+    // K in groups of 4, 2 or 1 chunks of 16 channels (rows of whole 128-pixel
+    // tiles: 1); the order of the sums, and so the result, depends on it
+    if (wd % 128 == 0) {
+        // three blocks of 32 or 64 output channels in one MMA: one of N = 32
+        // takes as long as one of N = 96
+        if constexpr (NT <= 64)
+            if (cout % (3 * NT) == 0)
+                return launch_conv_wide<NT, 3>(x, ct_in, kc, wt, bias, y, ct_out, cout, n, h, wd, relu, st);
+        return launch_conv_wide<NT, 1>(x, ct_in, kc, wt, bias, y, ct_out, cout, n, h, wd, relu, st);
+    }
+    if (kc % 4 == 0) return launch_conv_mt<NT, 1, 4, 1>(x, ct_in, kc, wt, bias, y, ct_out, cout, n, h, wd, relu, st);
+    if (kc % 2 == 0) return launch_conv_mt<NT, 1, 2, 1>(x, ct_in, kc, wt, bias, y, ct_out, cout, n, h, wd, relu, st);
+    return launch_conv_mt<NT, 1, 1, 1>(x, ct_in, kc, wt, bias, y, ct_out, cout, n, h, wd, relu, st);
 }
 
 template <int NT, int P, bool SW>
-int launch_wgrad_p(const void* x, int ct_x, int ci, const void* dy, int ct_dy, int co, float* dw, int h, int wd,
-                   int npix, long long total, cudaStream_t st)
+int launch_wgrad_p(const void* x, int ct_x, int ci, const void* dy, int ct_dy, int co, float* dw, int n, int h,
+                   int wd, cudaStream_t st)
 {
-    const int smem = smem_for_tmem(int(tmem_cols(3 * NT)), wgrad_smem_needed<NT, P, SW>());
+    constexpr int COT = wgrad_co_tile<NT, SW>(), CIT = wgrad_ci_tile<NT, SW>();
+    const int smem = smem_for_tmem(int(tmem_cols(9 * NT)), wgrad_smem_needed<NT, P, SW>());
     auto k = wgrad_tc_kernel<NT, P, SW>;
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return int(e);
-    constexpr int COT = wgrad_co_tile<NT, SW>(), CIT = wgrad_ci_tile<NT, SW>();
-    dim3 grid((co + COT - 1) / COT, (ci + CIT - 1) / CIT, int(3 * (total / npix)));
-    k<<<grid, kWgThreads, smem, st>>>((const bf16*)x, ct_x, ci, (const bf16*)dy, ct_dy, co, dw, h, wd, npix,
-                                      err_ptr());
-    return status(cudaGetLastError());
-}
-
-// CTAs of the weight gradient that fit on one SM (shared and tensor memory)
-template <int NT, int P, bool SW> int wgrad_ctas_per_sm()
-{
-    const int smem = smem_for_tmem(int(tmem_cols(3 * NT)), wgrad_smem_needed<NT, P, SW>());
-    const int by_smem = kSmemPerSm / (smem + 1024), by_tmem = 512 / int(tmem_cols(3 * NT));
-    return by_smem < by_tmem ? (by_smem > 0 ? by_smem : 1) : by_tmem;
-}
-
-template <int NT, int P, bool SW>
-int launch_wgrad_np(const void* x, int ct_x, int ci, const void* dy, int ct_dy, int co, float* dw, int n, int h,
-                    int wd, cudaStream_t st)
-{
-    // pixels per CTA: a power of two dividing the total, at most 4096 (long
-    // K loops: the tensor time of one layer is a few microseconds, and each
-    // split adds its co x ci x 3 partial sums into dw with atomics), halved
-    // while the grid fills less than half of the CTA slots, down to 8 K-steps
-    const long long total = (long long)n * h * wd;
+    const int tx = (co + COT - 1) / COT, ty = (ci + CIT - 1) / CIT;
+    const long long rows = (long long)n * (wd / P) * h;
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = at.val.clusterDim.y = 1;
+    cfg.blockDim = dim3(kWgThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    // clusters of the largest size that run at once on this device
+    at.val.clusterDim.z = kWgCluster;
+    cfg.gridDim = dim3(1, 1, kWgCluster);
+    static int at_once = 0;
+    if (at_once == 0) {
+        int c = 0;
+        if (cudaOccupancyMaxActiveClusters(&c, k, &cfg) != cudaSuccess || c < 1) {
+            cudaGetLastError();
+            c = 8;
+        }
+        at_once = c;
+    }
+    // One wave of CTAs that share the rows of all columns equally, at least 4
+    // rows each (a shorter CTA is mostly prologue and epilogue). Where that
+    // leaves SMs free, up to 8 CTAs form a cluster that adds its sums in a fixed
+    // order before the atomics, so that dw gets few addends (with at most two
+    // the result does not depend on their order). Clusters of 8 do not fill the
+    // SMs, so larger layers go without: 192 -> 64 channels at 32x128, 16 images,
+    // 41 us, with clusters 60.
     int sms = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, 0);
-    const long long slots = (long long)(sms > 0 ? sms : 148) * wgrad_ctas_per_sm<NT, P, SW>();
-    constexpr int COT = wgrad_co_tile<NT, SW>(), CIT = wgrad_ci_tile<NT, SW>();
-    const long long tiles = 3LL * ((co + COT - 1) / COT) * ((ci + CIT - 1) / CIT);
-    int npix = 4096;
-    while (npix > P && total % npix) npix >>= 1;
-    while (npix > 8 * P && tiles * (total / npix) < slots / 2 && total % (npix / 2) == 0) npix >>= 1;
-    return launch_wgrad_p<NT, P, SW>(x, ct_x, ci, dy, ct_dy, co, dw, h, wd, npix, total, st);
+    const long long most = (rows + 3) / 4, tiles = (long long)tx * ty;
+    const bool few = most * tiles <= (long long)at_once * kWgCluster;
+    long long splits = few ? most : (sms > 0 ? sms : 148) * (9 * NT <= 256 ? 2 : 1) / tiles;
+    if (splits > most) splits = most;
+    if (splits < 1) splits = 1;
+    int cs = 1;
+    while (few && cs < kWgCluster && 2 * cs <= splits) cs *= 2;
+    splits = splits / cs * cs;
+    const long long per = (rows + splits - 1) / splits;
+    at.val.clusterDim.z = cs;
+    cfg.gridDim = dim3(tx, ty, int(splits));
+    return status(cudaLaunchKernelEx(&cfg, k, (const bf16*)x, ct_x, ci, (const bf16*)dy, ct_dy, co, dw, h, wd, rows, per,
+                                     cs, err_ptr()));
 }
 
 template <int NT, bool SW>
 int launch_wgrad(const void* x, int ct_x, int ci, const void* dy, int ct_dy, int co, float* dw, int n, int h,
                  int wd, cudaStream_t st)
 {
-    // K-step: the widest of 64, 32, 16 pixels that divides the row (every
-    // step stays inside one image row)
-    if (wd % 64 == 0) return launch_wgrad_np<NT, 64, SW>(x, ct_x, ci, dy, ct_dy, co, dw, n, h, wd, st);
-    if (wd % 32 == 0) return launch_wgrad_np<NT, 32, SW>(x, ct_x, ci, dy, ct_dy, co, dw, n, h, wd, st);
-    return launch_wgrad_np<NT, 16, SW>(x, ct_x, ci, dy, ct_dy, co, dw, n, h, wd, st);
+    // columns of the widest of 64, 32 and 16 pixels that divides the row
+    if (wd % 64 == 0) return launch_wgrad_p<NT, 64, SW>(x, ct_x, ci, dy, ct_dy, co, dw, n, h, wd, st);
+    if (wd % 32 == 0) return launch_wgrad_p<NT, 32, SW>(x, ct_x, ci, dy, ct_dy, co, dw, n, h, wd, st);
+    return launch_wgrad_p<NT, 16, SW>(x, ct_x, ci, dy, ct_dy, co, dw, n, h, wd, st);
 }
 
 }  // namespace
@@ -1263,7 +1431,7 @@ int unet_conv3x3(const void* x, int ct_in, int cin, const void* wt, const float*
     // K runs over kc chunks of 16 channels: cin a multiple of 16, or cin < 16
     // in a view whose first 16 channels are readable (channels >= cin zero)
     const int kc = (cin + 15) / 16;
-    if (wd % kTileCols || h % kTileRows || cout % 32 || ct_in % 8 || ct_out % 8 || cin < 1 ||
+    if (wd % 32 || h % 4 || cout % 32 || ct_in % 8 || ct_out % 8 || cin < 1 ||
         (cin % 16 && cin > 16) || kc * 16 > ct_in ||
         (reinterpret_cast<uintptr_t>(x) | reinterpret_cast<uintptr_t>(y) | reinterpret_cast<uintptr_t>(wt)) & 15)
         return -1;
@@ -1282,23 +1450,10 @@ int unet_conv3x3_bwd_weight(const void* x, int ct_x, int ci, const void* dy, int
         (reinterpret_cast<uintptr_t>(x) | reinterpret_cast<uintptr_t>(dy)) & 15)
         return -1;
     cudaStream_t st = (cudaStream_t)stream;
-    // The MMA's 128 rows take the wider of the two channel counts: output
-    // channels (tiles of 128; input channels in N tiles of 128, 64, 32 or 16,
-    // at most ci rounded up to 16), or with more input than output channels
-    // (at most 128 of them) input channels (tiles of 128; output channels in
-    // one N tile of 32, 64 or 128).
+    // the wider of the two channel counts on the MMA's 128 rows
     int rc;
-    if (ci > co && co <= 128) {
-        if (co <= 32)
-            rc = launch_wgrad<32, true>(x, ct_x, ci, dy, ct_dy, co, dw, n, h, wd, st);
-        else if (co <= 64)
-            rc = launch_wgrad<64, true>(x, ct_x, ci, dy, ct_dy, co, dw, n, h, wd, st);
-        else
-            rc = launch_wgrad<128, true>(x, ct_x, ci, dy, ct_dy, co, dw, n, h, wd, st);
-    } else if (ci > 64)
-        rc = launch_wgrad<128, false>(x, ct_x, ci, dy, ct_dy, co, dw, n, h, wd, st);
-    else if (ci > 32)
-        rc = launch_wgrad<64, false>(x, ct_x, ci, dy, ct_dy, co, dw, n, h, wd, st);
+    if (ci > co)
+        rc = launch_wgrad<32, true>(x, ct_x, ci, dy, ct_dy, co, dw, n, h, wd, st);
     else if (ci > 16)
         rc = launch_wgrad<32, false>(x, ct_x, ci, dy, ct_dy, co, dw, n, h, wd, st);
     else
