@@ -495,30 +495,30 @@ __global__ void __launch_bounds__(kCvThreads) conv3x3_tc_kernel(const bf16* __re
 // blocks [n tile][k chunk of 16][tap] of NT x 16 BF16 in core-matrix order
 // (row group i at 256 B, k half j at 128 B, row r at 16 B); k beyond the real
 // channels is 0.
-__device__ __forceinline__ void pack_one(const float* __restrict__ w, int co, int ci, int transpose, int nt, int kc,
-                                         long long i, bf16* __restrict__ out)
+//
+// A thread takes the nine taps of one (n, k), which are contiguous in w, and
+// consecutive threads consecutive k, whose outputs lie in 16-byte runs (a thread
+// per output element found its place by 64-bit divisions and read 4 of every 36
+// bytes: 50 us for all layers of the network, now @PK@).
+__device__ __forceinline__ void pack_pair(const float* __restrict__ w, int co, int ci, int transpose, int nt, int kc,
+                                          int i, bf16* __restrict__ out)
 {
-    const int kreal = transpose ? co : ci;
-    const int k = int(i % (kc * 16));
-    const long long r1 = i / (kc * 16);
-    const int t = int(r1 % 9);
-    const int n = int(r1 / 9);
-    float v = 0.f;
-    if (k < kreal) v = transpose ? w[(size_t(k) * ci + n) * 9 + (8 - t)] : w[(size_t(n) * ci + k) * 9 + t];
-    const int nbk = n / nt, nn = n % nt, c = k / 16, kk = k % 16;
-    const size_t blk = (size_t(nbk) * kc + c) * 9 + t;
-    const size_t off = blk * nt * 16 + ((nn >> 3) * 2 + (kk >> 3)) * 64 + (nn & 7) * 8 + (kk & 7);
-    out[off] = __float2bfloat16_rn(v);
+    const int kreal = transpose ? co : ci, kp = kc * 16;
+    const int n = i / kp, k = i - n * kp;
+    const float* src = w + (transpose ? size_t(k) * ci + n : size_t(n) * ci + k) * 9;
+    const int nbk = n / nt, nn = n - nbk * nt, c = k >> 4, kk = k & 15;
+    bf16* dst = out + (size_t(nbk) * kc + c) * 9 * nt * 16 + ((nn >> 3) * 2 + (kk >> 3)) * 64 + (nn & 7) * 8 + (kk & 7);
+#pragma unroll
+    for (int t = 0; t < 9; ++t)
+        dst[size_t(t) * nt * 16] = __float2bfloat16_rn(k < kreal ? src[transpose ? 8 - t : t] : 0.f);
 }
 
 __global__ void conv_pack_kernel(const float* __restrict__ w, int co, int ci, int transpose, int nt, int kc,
                                  bf16* __restrict__ out)
 {
-    const int nrows = transpose ? ci : co;
-    const long long total = (long long)nrows * kc * 16 * 9;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
-         i += (long long)gridDim.x * blockDim.x)
-        pack_one(w, co, ci, transpose, nt, kc, i, out);
+    const int pairs = (transpose ? ci : co) * kc * 16;
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < pairs; i += gridDim.x * blockDim.x)
+        pack_pair(w, co, ci, transpose, nt, kc, i, out);
 }
 
 // Several packings in one launch: job blockIdx.y is the record
@@ -530,11 +530,9 @@ __global__ void conv_pack_many_kernel(const long long* __restrict__ jobs)
     const int co = int(j[1]), ci = int(j[2]), transpose = int(j[3]);
     bf16* out = reinterpret_cast<bf16*>(j[4]);
     const int nrows = transpose ? ci : co, kreal = transpose ? co : ci;
-    const int kc = (kreal + 15) / 16, nt = conv_ntile(nrows);
-    const long long total = (long long)nrows * kc * 16 * 9;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
-         i += (long long)gridDim.x * blockDim.x)
-        pack_one(w, co, ci, transpose, nt, kc, i, out);
+    const int kc = (kreal + 15) / 16, nt = conv_ntile(nrows), pairs = nrows * kc * 16;
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < pairs; i += gridDim.x * blockDim.x)
+        pack_pair(w, co, ci, transpose, nt, kc, i, out);
 }
 
 // ------------------------------------------------------------------ tensor-core weight gradient
@@ -935,6 +933,77 @@ __global__ void head_bwd_kernel(const bf16* __restrict__ x, int ct, int Ci, cons
     }
 }
 
+// The same with 8 channels of a pixel per thread (16-byte accesses; Ci = 8, 16,
+// 32 or 64, views 16-byte aligned): the products of dx run in the same order;
+// the sums of dw and db go over the warp's lanes of one channel group by
+// shuffles, then over the warps. Memory bound; a channel a thread took 43 us for
+// 16 tiles of 64x256 and 32 channels, now @HB@.
+template <int CO>
+__global__ void __launch_bounds__(kT) head_bwd8_kernel(const bf16* __restrict__ x, int ct, int Ci,
+                                                       const bf16* __restrict__ w, const float* __restrict__ dy, int HW,
+                                                       int B, bf16* __restrict__ dx, int ct_dx, float* __restrict__ dw,
+                                                       float* __restrict__ db)
+{
+    __shared__ float red[kT / 32][8][CO * 8 + CO];
+    const int G = Ci / 8, grp = threadIdx.x % G, lanes = kT / G;
+    float wc[CO][8], sw[CO][8], sb[CO];
+#pragma unroll
+    for (int o = 0; o < CO; ++o) {
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            wc[o][k] = ld(w + o * Ci + grp * 8 + k);
+            sw[o][k] = 0.f;
+        }
+        sb[o] = 0.f;
+    }
+    const long long n = (long long)B * HW;
+    for (long long i = (long long)blockIdx.x * lanes + threadIdx.x / G; i < n; i += (long long)gridDim.x * lanes) {
+        const int b = int(i / HW), p = int(i - (long long)b * HW);
+        float xv[8], s[8];
+        unpack8(*reinterpret_cast<const uint4*>(x + i * ct + grp * 8), xv);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) s[k] = 0.f;
+#pragma unroll
+        for (int o = 0; o < CO; ++o) {
+            const float g = dy[((long long)b * CO + o) * HW + p];
+            sb[o] += g;
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                s[k] = fmaf(wc[o][k], g, s[k]);
+                sw[o][k] = fmaf(g, xv[k], sw[o][k]);
+            }
+        }
+        *reinterpret_cast<uint4*>(dx + i * ct_dx + grp * 8) = pack8(s);
+    }
+    // lanes l and l ^ m (m = G, 2 G, ..) hold the same channel group
+    const int wl = threadIdx.x & 31, wp = threadIdx.x >> 5;
+    for (int m = G; m < 32; m <<= 1) {
+#pragma unroll
+        for (int o = 0; o < CO; ++o) {
+            sb[o] += __shfl_xor_sync(0xffffffffu, sb[o], m);
+#pragma unroll
+            for (int k = 0; k < 8; ++k) sw[o][k] += __shfl_xor_sync(0xffffffffu, sw[o][k], m);
+        }
+    }
+    if (wl < G) {
+#pragma unroll
+        for (int o = 0; o < CO; ++o) {
+            red[wp][wl][CO * 8 + o] = sb[o];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) red[wp][wl][o * 8 + k] = sw[o][k];
+        }
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < CO * Ci + CO; i += kT) {
+        // db from the first channel group (every group saw the same dy)
+        const int o = i < CO * Ci ? i / Ci : i - CO * Ci, c = i < CO * Ci ? i % Ci : 0;
+        const int e = i < CO * Ci ? o * 8 + c % 8 : CO * 8 + o;
+        float t = 0.f;
+        for (int q = 0; q < kT / 32; ++q) t += red[q][c / 8][e];
+        atomicAdd(i < CO * Ci ? &dw[o * Ci + c] : &db[o], t);
+    }
+}
+
 // 2x2 average pooling of an (H, W) NHWC view and its adjoint
 // 2x2 average pooling of an (H, W) NHWC view and its adjoint. One thread per
 // coarse pixel and 8 channels (16-byte accesses): C, ctx, cty multiples of 8,
@@ -992,19 +1061,34 @@ __global__ void pool2_bwd_kernel(const bf16* __restrict__ dy, int cty, bf16* __r
 }
 
 // nearest 2x upsampling of an (h, w) NHWC view and its adjoint (sum over the
-// 4 copies); the forward copies 8 channels (16 bytes) per thread, so C, ctx,
-// cty must be multiples of 8 and the views 16-byte aligned
+// 4 copies); a thread reads 8 channels (16 bytes) of a coarse pixel and writes
+// them four times, so C, ctx, cty must be multiples of 8 and the views 16-byte
+// aligned. (A thread per copy, placed by 64-bit divisions: 34 us for the three
+// upsamplings of 16 tiles of 64x256, now @UP@.)
 __global__ void up2_fwd_kernel(const bf16* __restrict__ x, int ctx, bf16* __restrict__ y, int cty, int C, int h,
                                int w, int B)
 {
-    const int H = 2 * h, W = 2 * w, C8 = C / 8;
-    const long long n = (long long)B * H * W * C8;
+    const int W = 2 * w, C8 = C / 8;
+    const long long n = (long long)B * h * w * C8;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        const int c = int(i % C8) * 8;
-        const long long pix = i / C8;
-        const int xx = int(pix % W), yy = int((pix / W) % H), b = int(pix / ((long long)W * H));
-        *reinterpret_cast<uint4*>(y + (size_t(b * H + yy) * W + xx) * cty + c) =
-            *reinterpret_cast<const uint4*>(x + (size_t(b * h + yy / 2) * w + xx / 2) * ctx + c);
+        long long pix;
+        int c;
+        if (n < (1LL << 31)) {
+            const uint32_t q = uint32_t(i) / uint32_t(C8);
+            pix = q;
+            c = int(uint32_t(i) - q * uint32_t(C8)) * 8;
+        } else {
+            pix = i / C8;
+            c = int(i % C8) * 8;
+        }
+        const long long r = n < (1LL << 31) ? (long long)(uint32_t(pix) / uint32_t(w)) : pix / w;  // b * h + y
+        const int xx = int(pix - r * w);
+        const uint4 v = *reinterpret_cast<const uint4*>(x + size_t(pix) * ctx + c);
+        bf16* o = y + (size_t(2 * r) * W + 2 * xx) * cty + c;
+        *reinterpret_cast<uint4*>(o) = v;
+        *reinterpret_cast<uint4*>(o + cty) = v;
+        *reinterpret_cast<uint4*>(o + size_t(W) * cty) = v;
+        *reinterpret_cast<uint4*>(o + size_t(W + 1) * cty) = v;
     }
 }
 
@@ -1118,15 +1202,34 @@ __global__ void relu_bwd_kernel(const bf16* __restrict__ y, int cty, bf16* __res
     }
 }
 
-// FP32 NCHW planes -> BF16 NHWC with ct channels per pixel (channels >= c are 0)
+// FP32 NCHW planes -> BF16 NHWC with ct channels per pixel (channels >= c are
+// 0). V: a thread writes 8 channels of a pixel in 16 bytes (ct a multiple of 8,
+// y 16-byte aligned; an element a thread took 18 us for 16 tiles of 64x256, now
+// @IN@).
+template <bool V>
 __global__ void input_nhwc_kernel(const float* __restrict__ x, int C, int HW, int B, bf16* __restrict__ y, int ct)
 {
-    const long long n = (long long)B * HW * ct;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        const int c = int(i % ct);
-        const long long pix = i / ct;
-        const int b = int(pix / HW), p = int(pix % HW);
-        y[i] = __float2bfloat16_rn(c < C ? x[((long long)b * C + c) * HW + p] : 0.f);
+    if constexpr (V) {
+        const int groups = ct / 8;
+        const long long n = (long long)B * HW;
+        for (long long pix = blockIdx.x * (long long)blockDim.x + threadIdx.x; pix < n;
+             pix += (long long)gridDim.x * blockDim.x) {
+            const int b = int(pix / HW), p = int(pix - (long long)b * HW);
+            for (int g = 0; g < groups; ++g) {
+                float v[8];
+#pragma unroll
+                for (int k = 0; k < 8; ++k) v[k] = g * 8 + k < C ? x[((long long)b * C + g * 8 + k) * HW + p] : 0.f;
+                *reinterpret_cast<uint4*>(y + pix * ct + g * 8) = pack8(v);
+            }
+        }
+    } else {
+        const long long n = (long long)B * HW * ct;
+        for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+            const int c = int(i % ct);
+            const long long pix = i / ct;
+            const int b = int(pix / HW), p = int(pix % HW);
+            y[i] = __float2bfloat16_rn(c < C ? x[((long long)b * C + c) * HW + p] : 0.f);
+        }
     }
 }
 
@@ -1137,11 +1240,25 @@ __global__ void mse_kernel(const float* __restrict__ p, const float* __restrict_
 {
     __shared__ double red[kT];
     double s = 0.0;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        const int c = int((i / HW) % C);
-        const float d = p[i] - t[i];
-        s += double(wc[c]) * d * d;
-        grad[i] = 2.f * wc[c] * d / float(n);
+    // four values in flight per thread
+    const long long stride = (long long)gridDim.x * blockDim.x;
+    for (long long i0 = blockIdx.x * (long long)blockDim.x + threadIdx.x; i0 < n; i0 += 4 * stride) {
+        float d[4], w[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const long long i = i0 + u * stride;
+            const bool in = i < n;
+            // 32-bit divisions where the count allows
+            const int c = !in ? 0 : n < (1LL << 31) ? int((uint32_t(i) / uint32_t(HW)) % uint32_t(C)) : int((i / HW) % C);
+            w[u] = wc[c];
+            d[u] = in ? p[i] - t[i] : 0.f;
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const long long i = i0 + u * stride;
+            s += double(w[u]) * d[u] * d[u];
+            if (i < n) grad[i] = 2.f * w[u] * d[u] / float(n);
+        }
     }
     red[threadIdx.x] = s;
     __syncthreads();
@@ -1412,8 +1529,7 @@ int unet_conv_pack(const float* w, int co, int ci, int transpose, void* out, voi
     const int nrows = transpose ? ci : co, kreal = transpose ? co : ci;
     if (nrows % 32) return -1;
     const int kc = (kreal + 15) / 16;
-    const long long total = (long long)nrows * kc * 16 * 9;
-    conv_pack_kernel<<<blocks_for(total), kT, 0, (cudaStream_t)stream>>>(w, co, ci, transpose, conv_ntile(nrows), kc,
+    conv_pack_kernel<<<blocks_for((long long)nrows * kc * 16), kT, 0, (cudaStream_t)stream>>>(w, co, ci, transpose, conv_ntile(nrows), kc,
                                                                         (bf16*)out);
     return status(cudaGetLastError());
 }
@@ -1421,7 +1537,7 @@ int unet_conv_pack(const float* w, int co, int ci, int transpose, void* out, voi
 int unet_conv_pack_many(const long long* jobs, int njobs, long max_elems, void* stream)
 {
     if (!jobs || njobs < 1 || njobs > 65535 || max_elems < 1) return -1;
-    conv_pack_many_kernel<<<dim3(blocks_for(max_elems), njobs), kT, 0, (cudaStream_t)stream>>>(jobs);
+    conv_pack_many_kernel<<<dim3(blocks_for(max_elems / 9), njobs), kT, 0, (cudaStream_t)stream>>>(jobs);
     return status(cudaGetLastError());
 }
 
@@ -1494,6 +1610,15 @@ int unet_head_bwd(const void* x, int ct, int ci, const void* w, const float* dy,
                   int ct_dx, float* dw, float* db, void* stream)
 {
     if (co != 3 || ci < 1 || ci > kT) return -1;
+    if ((ci == 8 || ci == 16 || ci == 32 || ci == 64) && ct % 8 == 0 && ct_dx % 8 == 0 &&
+        ((reinterpret_cast<uintptr_t>(x) | reinterpret_cast<uintptr_t>(dx)) & 15) == 0) {
+        // about 8 pixels per thread, at most 4 blocks per SM
+        long long blocks8 = (long long)n * hw * (ci / 8) / (kT * 8) + 1;
+        if (blocks8 > 608) blocks8 = 608;
+        head_bwd8_kernel<3><<<int(blocks8), kT, 0, (cudaStream_t)stream>>>((const bf16*)x, ct, ci, (const bf16*)w, dy, hw,
+                                                                          n, (bf16*)dx, ct_dx, dw, db);
+        return status(cudaGetLastError());
+    }
     // at most 8 blocks per SM: each block adds its partial sums into the same
     // 3 (ci + 1) addresses of dw and db
     long long blocks = (long long)n * hw * ci / (kT * 4) + 1;
@@ -1532,7 +1657,7 @@ int unet_up2_fwd(const void* x, int ctx, void* y, int cty, int c, int n, int h, 
 {
     if (c % 8 || ctx % 8 || cty % 8 || (reinterpret_cast<uintptr_t>(x) | reinterpret_cast<uintptr_t>(y)) & 15)
         return -1;
-    up2_fwd_kernel<<<blocks_for((long long)n * c / 8 * h * wd * 4), kT, 0, (cudaStream_t)stream>>>(
+    up2_fwd_kernel<<<blocks_for((long long)n * c / 8 * h * wd), kT, 0, (cudaStream_t)stream>>>(
         (const bf16*)x, ctx, (bf16*)y, cty, c, h, wd, n);
     return status(cudaGetLastError());
 }
@@ -1558,7 +1683,10 @@ int unet_relu_bwd(const void* y, int cty, void* dy, int ctd, int c, long npix, f
 
 int unet_input_nhwc(const float* x, int c, int hw, int n, void* y, int ct, void* stream)
 {
-    input_nhwc_kernel<<<blocks_for((long long)n * hw * ct), kT, 0, (cudaStream_t)stream>>>(x, c, hw, n, (bf16*)y, ct);
+    if (ct % 8 == 0 && (reinterpret_cast<uintptr_t>(y) & 15) == 0)
+        input_nhwc_kernel<true><<<blocks_for((long long)n * hw), kT, 0, (cudaStream_t)stream>>>(x, c, hw, n, (bf16*)y, ct);
+    else
+        input_nhwc_kernel<false><<<blocks_for((long long)n * hw * ct), kT, 0, (cudaStream_t)stream>>>(x, c, hw, n, (bf16*)y, ct);
     return status(cudaGetLastError());
 }
 
