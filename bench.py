@@ -522,7 +522,7 @@ def storage_forms(lbm, stream, w, params, steps=50):
 
 def small_configs(lbm, stream):
     """The 128x64 sessile droplet and the 1024x128 rough channel as single
-    domains (launch-bound, L2-resident: one kernel launch per step), and the
+    domains (on the chip for many steps per launch), and the
     rough channel's steady flux Q(f)/Q(0) at four force levels, run to steady
     as one batch (FP32 deviation storage)."""
     import torch

@@ -10,8 +10,8 @@
 // of each step: a launch, the staging of the first rows, the row pipeline. Here
 // a step is two CTA barriers, and the launch, the staging and the trip of the
 // whole state through L2 fall away. Measured (us per step, before -> now):
-// 128x64 FP32 6.7 -> 0.95, 1024x128 FP32 deviations 8.2 -> 2.6 (6.9 -> 2.3 in
-// FP32), 1024x256 FP16 deviations 8.3 -> 4.1, 1024x512 FP32 11.0 -> 5.3.
+// 128x64 FP32 6.7 -> 0.9, 1024x128 FP32 deviations 8.2 -> 2.8 (8.2 -> 2.3 in
+// FP32), 1024x256 FP16 deviations 8.5 -> 4.1, 1024x512 FP32 11.0 -> 5.3.
 //
 // A round is K steps and one exchange. The tile holds a halo of 2 K nodes (a
 // step reaches two nodes: one for the pull, one for psi); step m of the round
