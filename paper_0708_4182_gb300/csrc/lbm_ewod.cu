@@ -1030,12 +1030,17 @@ const void* resident_fn(int storage, bool t1, int j, bool batch)
     }
 }
 
-// Allow the launch shape of a plan; false if its CTAs would not be resident
-// together on this device.
+// Whether a plan's CTAs would be resident together on this device. The kernel
+// instance is allowed all the shared memory a CTA can have, not the plan's: the
+// limit belongs to the instance, which contexts and groups with other plans
+// share (a plan that set its own would take it from a larger one still in use).
 bool resident_fits(const void* fn, const ResPlan& r, int ctas, int sm_count)
 {
     int per_sm = 0;
-    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, int(r.smem)) != cudaSuccess ||
+    cudaFuncAttributes at{};
+    if (cudaFuncGetAttributes(&at, fn) != cudaSuccess || r.smem + at.sharedSizeBytes > kResSmemCta ||
+        cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kResSmemCta - at.sharedSizeBytes)) !=
+            cudaSuccess ||
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, r.nt, r.smem) != cudaSuccess) {
         cudaGetLastError();
         return false;
