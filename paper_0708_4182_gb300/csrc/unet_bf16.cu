@@ -768,12 +768,13 @@ __global__ void __launch_bounds__(kWgThreads) wgrad_tc_kernel(const bf16* __rest
                 red[SW ? (n0 + c) * RP + m * 9 + t : m * RP + (n0 + c) * 9 + t] = ok ? v[t][c] : 0.f;
             }
     }
+    // Tensor memory goes back before any wait for the cluster: a peer may still
+    // wait for its own allocation, behind a CTA of another launch that holds the
+    // columns and waits for a peer in its turn.
     tc_fence_before();
-    if (cs > 1)
-        cluster_sync();
-    else
-        __syncthreads();
+    __syncthreads();
     if (warp == 0) tmem_dealloc(tmem, kCols);
+    if (cs > 1) cluster_sync();
     const int len = ci_here * 9;
     if (cs == 1) {
         // a warp per output channel
