@@ -29,6 +29,7 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <atomic>
 #include <cstdint>
 
 namespace unet {
@@ -1404,8 +1405,18 @@ int launch_conv_mt(const void* x, int ct_in, int kc, const void* wt, const float
         ++wslots;
     const int smem = smem_for_tmem(cols, int(conv_smem<NT, NG, CK, MT>(S, wslots)));
     auto k = conv3x3_tc_kernel<NT, NG, CK, MT>;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e != cudaSuccess) return int(e);
+    // the instance's limit, the same in every call (not this width's need): calls
+    // of other widths may run in other threads
+    static std::atomic<int> known{0};
+    int limit = known.load(std::memory_order_relaxed);
+    cudaError_t e = cudaSuccess;
+    if (limit == 0) {
+        cudaFuncAttributes at{};
+        if ((e = cudaFuncGetAttributes(&at, k)) != cudaSuccess) return int(e);
+        limit = kSmemPerSm - 1024 - int(at.sharedSizeBytes);
+        known.store(limit, std::memory_order_relaxed);
+    }
+    if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, limit)) != cudaSuccess) return int(e);
     dim3 grid((wd / S) * ((h * (S + 2) + 128 * MT - 1) / (128 * MT)), cout / (NT * NG), n);
     k<<<grid, kCvThreads, smem, st>>>((const bf16*)x, ct_in, kc, (const bf16*)wt, bias, (bf16*)y, ct_out, h, wd, S,
                                       relu, wslots, err_ptr());
