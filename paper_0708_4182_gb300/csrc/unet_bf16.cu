@@ -1483,14 +1483,21 @@ int launch_wgrad_p(const void* x, int ct_x, int ci, const void* dy, int ct_dy, i
     // clusters of the largest size that run at once on this device
     at.val.clusterDim.z = kWgCluster;
     cfg.gridDim = dim3(1, 1, kWgCluster);
-    static int at_once = 0;
+    int dev = 0, sms = 0, at_once = 0;
+    if ((e = cudaGetDevice(&dev)) != cudaSuccess ||
+        (e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
+        return int(e);
+    // known per device; a query that fails is asked again, and the call goes
+    // without clusters
+    constexpr int kDevices = 32;
+    static std::atomic<int> known[kDevices];
+    if (dev < kDevices) at_once = known[dev].load(std::memory_order_relaxed);
     if (at_once == 0) {
-        int c = 0;
-        if (cudaOccupancyMaxActiveClusters(&c, k, &cfg) != cudaSuccess || c < 1) {
+        if (cudaOccupancyMaxActiveClusters(&at_once, k, &cfg) != cudaSuccess || at_once < 0) {
             cudaGetLastError();
-            c = 8;
+            at_once = 0;
         }
-        at_once = c;
+        if (dev < kDevices) known[dev].store(at_once, std::memory_order_relaxed);
     }
     // Whole waves of CTAs (mostly one) that share the rows of all columns equally,
     // at least 4 rows each (a shorter CTA is mostly prologue and epilogue). Where that
@@ -1499,11 +1506,9 @@ int launch_wgrad_p(const void* x, int ct_x, int ci, const void* dy, int ct_dy, i
     // the result does not depend on their order). Clusters of 8 do not fill the
     // SMs, so larger layers go without: 192 -> 64 channels at 32x128, 16 images,
     // 41 us, with clusters 60.
-    int sms = 0;
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, 0);
     const long long most = (rows + 3) / 4, tiles = (long long)tx * ty;
     const bool few = most * tiles <= (long long)at_once * kWgCluster;
-    const long long wave = (sms > 0 ? sms : 148) * (9 * NT <= 256 ? 2 : 1) / tiles;
+    const long long wave = sms * (9 * NT <= 256 ? 2 : 1) / tiles;
     long long splits = few ? most : wave;
     if (splits > most) splits = most;
     if (splits < 1) splits = 1;
