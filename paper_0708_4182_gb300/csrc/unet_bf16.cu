@@ -1264,8 +1264,9 @@ __global__ void mse_kernel(const float* __restrict__ p, const float* __restrict_
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
             const long long i = i0 + u * stride;
+            if (i >= n) continue;  // (an infinite weight times the padding's 0 would be NaN)
             s += double(w[u]) * d[u] * d[u];
-            if (i < n) grad[i] = 2.f * w[u] * d[u] / float(n);
+            grad[i] = 2.f * w[u] * d[u] / float(n);
         }
     }
     red[threadIdx.x] = s;
