@@ -1073,12 +1073,29 @@ bool capturing(cudaStream_t st)
 }
 
 // Steps per resident launch at most: about a millisecond or two, so that
-// other streams' work gets its turn.
+// other streams' work gets its turn. Even, so that only a call's last launch
+// can have an odd number of steps.
 constexpr int kResChunk = 1024;
+static_assert(kResChunk % 2 == 0, "an even number of steps returns the state to its buffer");
 // Fewer steps are launched one by one: a resident launch loads and stores the
 // state once more. Measured (us for 2 and 3 steps, resident / one by one):
 // 128x64 8.6 and 9.8 / 16.7 and 24.8; 1024x512 30 and 36 / 29 and 43.
 constexpr int kResMinSteps = 2;
+
+// The next launch of `left` steps: n of them, with an exchange every k. An even
+// number of steps leaves the state in the buffer where it was, as steps one by
+// one do, so that a captured even number of steps stays valid between calls: it
+// runs in place, which needs at least one exchange.
+struct ResLaunch {
+    int n, k;
+    bool swap;
+};
+ResLaunch resident_launch(int64_t left, int k)
+{
+    const int n = int(std::min<int64_t>(left, kResChunk));
+    const bool swap = n % 2 != 0;
+    return {n, swap || n > k ? k : n / 2, swap};
+}
 
 // nsteps plain steps of a domain that fits on the chip. *done = false if this
 // device cannot hold the launch right now (the caller steps one by one).
@@ -1088,14 +1105,14 @@ lbm_status resident_steps(lbm_ctx* c, int64_t nsteps, bool* done)
     const void* fn = resident_fn(c->prm.storage, c->ph.tau == 1.f, r.j, false);
     *done = true;
     while (nsteps > 0) {
-        int n = int(std::min<int64_t>(nsteps, kResChunk));
+        ResLaunch l = resident_launch(nsteps, r.k);
         const float* in = c->cur;
-        float* out = c->nxt;
-        int tx = r.tx, ty = r.ty, k = r.k, cap = r.edge_cap, stride = int(c->L.exch_bytes / 2 / sizeof(uint4));
+        float* out = l.swap ? c->nxt : c->cur;
+        int tx = r.tx, ty = r.ty, cap = r.edge_cap, stride = int(c->L.exch_bytes / 2 / sizeof(uint4));
         uint32_t tag = 0;
-        lbm_status s = take_tags(&c->res_tag, n, c->exch, c->L.exch_bytes, c->stream, &tag);
+        lbm_status s = take_tags(&c->res_tag, l.n, c->exch, c->L.exch_bytes, c->stream, &tag);
         if (s) return fail(c, s, "exchange buffer clear");
-        void* args[] = {&in, &out, &c->g, &c->ph, &tx, &ty, &k, &c->exch, &stride, &cap, &tag, &n, &c->status};
+        void* args[] = {&in, &out, &c->g, &c->ph, &tx, &ty, &l.k, &c->exch, &stride, &cap, &tag, &l.n, &c->status};
         const cudaError_t e = cudaLaunchCooperativeKernel(fn, dim3(r.tiles()), dim3(r.nt), args, r.smem, c->stream);
         if (e == cudaErrorCooperativeLaunchTooLarge) {
             cudaGetLastError();
@@ -1104,9 +1121,9 @@ lbm_status resident_steps(lbm_ctx* c, int64_t nsteps, bool* done)
             return LBM_OK;
         }
         if ((s = check_cuda(c, e, "resident steps launch"))) return s;
-        c->t += n;
-        std::swap(c->cur, c->nxt);
-        nsteps -= n;
+        c->t += l.n;
+        if (l.swap) std::swap(c->cur, c->nxt);
+        nsteps -= l.n;
     }
     return LBM_OK;
 }
@@ -2106,33 +2123,32 @@ lbm_status resident_batch_steps(lbm_batch* b, int64_t nsteps, bool* done)
     // by a clear margin: for large sweeps the two are within the estimates' error
     // (64 uneven channels, 11.7 M nodes: 11.6 ms resident, 11.4 ms by the walk)
     if (b->groups.empty() || 1.3 * (b->res_us * double(nsteps) + b->res_us_once) >= b->walk_us * double(nsteps)) return LBM_OK;
-    int launches = 0;
     for (const lbm_batch::Group& gr : b->groups) {
         const void* fn = resident_fn(b->storage, b->tau1, gr.plan.j, true);
         const int2* ctas = b->d_ctas + gr.first;
-        int k = gr.plan.k, cap = gr.plan.edge_cap, stride = gr.ctas * res_records(b->storage) * cap;
-        launches = 0;
-        for (int64_t left = nsteps; left > 0; ++launches) {
-            int n = int(std::min<int64_t>(left, kResChunk)), parity = launches & 1;
+        int cap = gr.plan.edge_cap, stride = gr.ctas * res_records(b->storage) * cap;
+        for (int64_t left = nsteps; left > 0;) {
+            ResLaunch l = resident_launch(left, gr.plan.k);
+            int in = 0, out = l.swap ? 1 : 0;  // (a swapping launch is the last)
             uint32_t tag = 0;
-            if ((s = take_tags(&b->res_tag, n, b->exch, b->exch_bytes, b->stream, &tag)))
+            if ((s = take_tags(&b->res_tag, l.n, b->exch, b->exch_bytes, b->stream, &tag)))
                 return bfail(b, s, "exchange buffer clear");
-            void* args[] = {&b->d_dom, &b->d_shape, &ctas, &parity, &k, &b->exch, &stride, &cap, &tag, &n, &b->d_status};
+            void* args[] = {&b->d_dom, &b->d_shape, &ctas, &in, &out, &l.k, &b->exch, &stride, &cap, &tag, &l.n, &b->d_status};
             const cudaError_t e = cudaLaunchCooperativeKernel(fn, dim3(gr.ctas), dim3(gr.plan.nt), args, gr.plan.smem, b->stream);
-            if (e == cudaErrorCooperativeLaunchTooLarge && launches == 0 && &gr == &b->groups.front()) {
+            if (e == cudaErrorCooperativeLaunchTooLarge && left == nsteps && &gr == &b->groups.front()) {
                 cudaGetLastError();
                 b->res_allowed = false;
                 return LBM_OK;
             }
             if ((s = bcheck(b, e, "resident steps launch"))) return s;
-            left -= n;
+            left -= l.n;
         }
     }
     for (int d = 0; d < b->count; ++d) {
         if (!b->active[d]) continue;
         lbm_ctx* c = b->ctx[d];
         c->t += nsteps;
-        if (launches & 1) std::swap(c->cur, c->nxt);
+        if (nsteps & 1) std::swap(c->cur, c->nxt);
     }
     *done = true;
     return LBM_OK;

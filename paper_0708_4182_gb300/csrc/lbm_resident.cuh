@@ -294,10 +294,12 @@ template <int ST> __device__ __forceinline__ void put_node_records(uint4* q, int
 
 // nsteps steps of one tile, a halo of 2 K nodes exchanged every K steps (the
 // last round may be shorter). J: rows per warp at most. exch: 2 x (CTAs of
-// the launch) x records x edge_cap records.
+// the launch) x records x edge_cap records. out may be in where the launch has
+// an exchange (nsteps > K): a tile writes its final state after it has received
+// records from every tile that reads it, which those publish after their loads.
 template <int ST, bool T1, int J>
-__device__ __forceinline__ void run_resident(const Geom& g, const Phys& p, const float* __restrict__ in,
-                                             float* __restrict__ out, int tx, int ty, int first, int tile, int K,
+__device__ __forceinline__ void run_resident(const Geom& g, const Phys& p, const float* in,
+                                             float* out, int tx, int ty, int first, int tile, int K,
                                              uint4* exch, int parity_stride, int edge_cap, uint32_t tag0, int nsteps,
                                              int* err, unsigned char* smem)
 {
@@ -497,7 +499,7 @@ __device__ __forceinline__ void run_resident(const Geom& g, const Phys& p, const
 // One domain, every CTA one tile.
 template <int ST, bool T1, int J>
 __global__ void __launch_bounds__(res_max_threads(J), 2)
-    resident_kernel(const float* __restrict__ in, float* __restrict__ out, Geom g, Phys p, int tx, int ty, int K,
+    resident_kernel(const float* in, float* out, Geom g, Phys p, int tx, int ty, int K,
                     uint4* exch, int parity_stride, int edge_cap, uint32_t tag0, int nsteps, int* err)
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -506,11 +508,12 @@ __global__ void __launch_bounds__(res_max_threads(J), 2)
 }
 
 // Several domains: CTA i works on tile ctas[i].y of domain ctas[i].x, whose
-// tiling is shape (tx, ty, first CTA); buffers as in batch_step_kernel.
+// tiling is shape (tx, ty, first CTA); buf[parity] is read and buf[parity_out]
+// written.
 template <int ST, bool T1, int J>
 __global__ void __launch_bounds__(res_max_threads(J), 2)
     resident_batch_kernel(const DomainDev* __restrict__ doms, const int4* __restrict__ shape,
-                          const int2* __restrict__ ctas, int parity, int K, uint4* exch, int parity_stride,
+                          const int2* __restrict__ ctas, int parity, int parity_out, int K, uint4* exch, int parity_stride,
                           int edge_cap, uint32_t tag0, int nsteps, int* err)
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -524,7 +527,7 @@ __global__ void __launch_bounds__(res_max_threads(J), 2)
     }
     __syncthreads();
     const int4 sh = shape[c.x];
-    run_resident<ST, T1, J>(g, p, d.buf[parity], d.buf[parity ^ 1], sh.x, sh.y, sh.z, c.y, K, exch, parity_stride,
+    run_resident<ST, T1, J>(g, p, d.buf[parity], d.buf[parity_out], sh.x, sh.y, sh.z, c.y, K, exch, parity_stride,
                             edge_cap, tag0, nsteps, err, smem_raw);
 }
 
