@@ -210,6 +210,10 @@ lbm_status lbm_get_field(lbm_ctx *ctx, int which, double *out, int on_device);
  * are set. */
 lbm_status lbm_step(lbm_ctx *ctx, int64_t nsteps);
 
+/* Launches of the resident kernel on this context so far (-1 for NULL): which
+ * way lbm_step went, for tests and tuning. */
+int64_t lbm_resident_launches(const lbm_ctx *ctx);
+
 /* Self-test of the device-side timeout path (no counterpart in the paper):
  * one kernel waits, with the step kernel's bounded mbarrier wait (2^18
  * polls), on an mbarrier phase that nothing completes. The wait gives up and
@@ -289,6 +293,11 @@ lbm_ctx *lbm_batch_domain(lbm_batch *b, int32_t i);
  * persistent kernel whose CTAs walk a tile list (domain, strip, row segment)
  * covering all active domains; pairs of steps run as one CUDA graph. */
 lbm_status lbm_batch_step(lbm_batch *b, int64_t nsteps);
+
+/* Launches of the resident kernel for this batch so far, and the groups (one
+ * launch each) of the last resident call's domains; -1 for NULL. */
+int64_t lbm_batch_resident_launches(const lbm_batch *b);
+int32_t lbm_batch_resident_groups(const lbm_batch *b);
 
 /* Observables of every domain (one batched pass), out[count]. */
 lbm_status lbm_batch_observables(lbm_batch *b, lbm_obs *out);

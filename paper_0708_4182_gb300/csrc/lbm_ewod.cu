@@ -808,6 +808,7 @@ struct lbm_ctx {
     cudaGraphExec_t step_graph[2] = {nullptr, nullptr};
     uint4* exch = nullptr;  // exchange records of the resident kernel (NULL: not used)
     uint32_t res_tag = 1;   // next unused tag
+    int64_t res_launches = 0;
     ~lbm_ctx()
     {
         for (cudaGraphExec_t e : step_graph)
@@ -1121,6 +1122,7 @@ lbm_status resident_steps(lbm_ctx* c, int64_t nsteps, bool* done)
             return LBM_OK;
         }
         if ((s = check_cuda(c, e, "resident steps launch"))) return s;
+        ++c->res_launches;
         c->t += l.n;
         if (l.swap) std::swap(c->cur, c->nxt);
         nsteps -= l.n;
@@ -1591,6 +1593,8 @@ lbm_status lbm_obs_latest_async(lbm_ctx* c, lbm_obs* out)
 
 int64_t lbm_time(const lbm_ctx* c) { return c ? c->t : -1; }
 
+int64_t lbm_resident_launches(const lbm_ctx* c) { return c ? c->res_launches : -1; }
+
 const char* lbm_last_error(const lbm_ctx* c) { return c ? c->err : "null context"; }
 
 const char* lbm_status_string(int s)
@@ -1778,6 +1782,7 @@ struct lbm_batch {
     uint4* exch = nullptr;
     size_t exch_bytes = 0;
     uint32_t res_tag = 1;
+    int64_t res_launches = 0;
     int4* d_shape = nullptr;             // per domain: tx, ty, first CTA of its group's launch
     int2* d_ctas = nullptr;              // (domain, tile) of every CTA
     std::vector<int4> h_shape;
@@ -2141,6 +2146,7 @@ lbm_status resident_batch_steps(lbm_batch* b, int64_t nsteps, bool* done)
                 return LBM_OK;
             }
             if ((s = bcheck(b, e, "resident steps launch"))) return s;
+            ++b->res_launches;
             left -= l.n;
         }
     }
@@ -2365,6 +2371,10 @@ lbm_status lbm_batch_step(lbm_batch* b, int64_t nsteps)
     }
     return LBM_OK;
 }
+
+int64_t lbm_batch_resident_launches(const lbm_batch* b) { return b ? b->res_launches : -1; }
+
+int32_t lbm_batch_resident_groups(const lbm_batch* b) { return b ? int32_t(b->groups.size()) : -1; }
 
 lbm_status lbm_batch_observables(lbm_batch* b, lbm_obs* out)
 {

@@ -7,7 +7,7 @@ workspace tensor) and for the CUDA stream the context enqueues on.
 
 Low level: ``lbm_workspace_bytes``, ``lbm_create``, ``lbm_set_geometry``,
 ``lbm_set_field``, ``lbm_set_density_f32``, ``lbm_get_field``, ``lbm_step``, ``lbm_observables``,
-``lbm_obs_latest``, ``lbm_obs_latest_async``, ``lbm_time``, ``lbm_last_error``, ``lbm_status_string``,
+``lbm_obs_latest``, ``lbm_obs_latest_async``, ``lbm_time``, ``lbm_resident_launches``, ``lbm_last_error``, ``lbm_status_string``,
 ``lbm_destroy``; each raises ``LbmError`` on a non-zero status.
 High level: ``Lattice`` owns a workspace tensor and a context.
 """
@@ -93,6 +93,7 @@ def load():
             "lbm_obs_latest_async": (ctypes.c_int, [vp, vp]),
             "lbm_run_to_steady": (ctypes.c_int, [vp, ctypes.c_double, ctypes.c_int64, ctypes.c_int64, O]),
             "lbm_time": (ctypes.c_int64, [vp]),
+            "lbm_resident_launches": (ctypes.c_int64, [vp]),
             "lbm_selftest_timeout": (ctypes.c_int, [vp]),
             "lbm_last_error": (ctypes.c_char_p, [vp]),
             "lbm_status_string": (ctypes.c_char_p, [ctypes.c_int]),
@@ -202,6 +203,10 @@ def lbm_run_to_steady(ctx, rel_tol: float, check_every: int, max_steps: int) -> 
 
 def lbm_time(ctx) -> int:
     return int(load().lbm_time(ctx))
+
+
+def lbm_resident_launches(ctx) -> int:
+    return int(load().lbm_resident_launches(ctx))
 
 
 def lbm_last_error(ctx) -> str:
@@ -371,6 +376,11 @@ class Lattice:
     def time(self) -> int:
         return lbm_time(self.ctx)
 
+    @property
+    def resident_launches(self) -> int:
+        """Launches of the resident kernel so far (many steps each)."""
+        return lbm_resident_launches(self.ctx)
+
     def close(self):
         if getattr(self, "ctx", None) and getattr(self, "_owner", None) is None:
             lbm_destroy(self.ctx)
@@ -424,6 +434,8 @@ def _batch_lib():
             "lbm_batch_create": (ctypes.c_int, [P, ctypes.c_int32, vp, ctypes.c_size_t, vp, ctypes.POINTER(vp)]),
             "lbm_batch_domain": (vp, [vp, ctypes.c_int32]),
             "lbm_batch_step": (ctypes.c_int, [vp, ctypes.c_int64]),
+            "lbm_batch_resident_launches": (ctypes.c_int64, [vp]),
+            "lbm_batch_resident_groups": (ctypes.c_int32, [vp]),
             "lbm_batch_observables": (ctypes.c_int, [vp, O]),
             "lbm_batch_set_active": (ctypes.c_int, [vp, ctypes.POINTER(ctypes.c_uint8)]),
             "lbm_batch_set_tile_rows": (ctypes.c_int, [vp, ctypes.c_int32]),
@@ -488,6 +500,15 @@ class Batch:
 
     def step(self, n: int = 1):
         self._check(_batch_lib().lbm_batch_step(self.handle, int(n)))
+
+    @property
+    def resident_launches(self) -> int:
+        """Launches of the resident kernel so far (many steps each)."""
+        return int(_batch_lib().lbm_batch_resident_launches(self.handle))
+
+    @property
+    def resident_groups(self) -> int:
+        return int(_batch_lib().lbm_batch_resident_groups(self.handle))
 
     def observables(self, check_finite: bool = True) -> list:
         """Per-domain observables; a non-finite domain raises unless

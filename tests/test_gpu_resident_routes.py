@@ -1,0 +1,89 @@
+"""Which calls run in the resident kernel: the comparisons with the step kernel
+mean nothing where both sides take the same way."""
+import numpy as np
+import pytest
+from test_gpu_resident import CASES, domain
+
+from paper_0708_4182_gb300 import workloads as wl
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def lbm():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_0708_4182_gb300 import lbm as L
+    L.load()
+    return L
+
+
+def ready(lbm, nx, ny, **more):
+    p = dict(wl.PAPER, f_elec=0.1, body_fx=1e-5, **more)
+    lat = lbm.Lattice(nx, ny, **p)
+    mask, rho = domain(nx, ny, True, 1)
+    lat.set_geometry(mask)
+    lat.set_rho(np.where(mask, 0.0, 1.5 + 0 * rho))
+    return lat
+
+
+@pytest.mark.parametrize("nx,ny,walls,storage,tau", CASES)
+def test_compared_domains_are_resident(lbm, nx, ny, walls, storage, tau):
+    lat = ready(lbm, nx, ny, storage=storage, tau=tau)
+    lat.step(9)
+    assert lat.resident_launches == 1
+    lat.step(1)
+    assert lat.resident_launches == 1  # a single step is a launch of its own
+
+
+@pytest.mark.parametrize("more", [
+    dict(layout=1), dict(layout=2), dict(tile_rows=8), dict(obs_every=1), dict(nx=1024, ny=900), dict(nx=1024, ny=512, tau=0.9),
+])
+def test_other_calls_are_not(lbm, more):
+    more = dict(more)
+    lat = ready(lbm, more.pop("nx", 128), more.pop("ny", 64), **more)
+    lat.step(40)
+    lat.observables()
+    assert lat.resident_launches == 0
+
+
+def test_captured_steps_are_not(lbm):
+    import torch
+    st = torch.cuda.Stream()
+    lat = lbm.Lattice(128, 64, stream=st, **wl.PAPER)
+    mask, _ = domain(128, 64, True, 1)
+    lat.set_geometry(mask)
+    lat.set_rho(np.where(mask, 0.0, 1.5))
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=st):
+        lat.step(6)
+    assert lat.resident_launches == 0
+    lat.step(6)
+    assert lat.resident_launches == 1
+
+
+@pytest.mark.parametrize("tau,sizes,groups", [
+    (1.0, ((256, 64), (40, 30), (320, 200), (64, 4), (8, 100), (264, 61), (512, 256)), 1),
+    (0.9, ((514, 297), (575, 171), (429, 188)), 2), (1.0, ((1011, 132), (773, 554)), 2),
+])
+def test_batches(lbm, tau, sizes, groups):
+    p = dict(wl.PAPER, tau=tau, storage=lbm.LBM_FP32_DEV)
+    for more, resident in ((dict(), True), (dict(layout=lbm.LBM_LAYOUT_SINGLE), False), (dict(tile_rows=16), False)):
+        b = lbm.Batch([dict(nx=nx, ny=ny, **p, **more) for nx, ny in sizes])
+        for (nx, ny), d in zip(sizes, b.domains):
+            mask, _ = domain(nx, ny, True, nx)
+            d.set_geometry(mask)
+            d.set_rho(np.where(mask, 0.0, 1.5))
+        b.step(50)
+        b.observables()
+        assert (b.resident_groups, b.resident_launches) == ((groups, groups) if resident else (0, 0))
+
+
+def test_larger_plans_stay_resident(lbm):
+    lats = [ready(lbm, nx, ny, storage=lbm.LBM_FP32_DEV) for nx, ny in ((2048, 256), (1024, 512), (640, 400), (128, 64), (301, 67))]
+    for lat in lats:
+        lat.step(20)
+        lat.observables()
+        assert lat.resident_launches == 1
