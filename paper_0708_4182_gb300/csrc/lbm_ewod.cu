@@ -1078,10 +1078,20 @@ bool capturing(cudaStream_t st)
 // can have an odd number of steps.
 constexpr int kResChunk = 1024;
 static_assert(kResChunk % 2 == 0, "an even number of steps returns the state to its buffer");
-// Fewer steps are launched one by one: a resident launch loads and stores the
-// state once more. Measured (us for 2 and 3 steps, resident / one by one):
-// 128x64 8.6 and 9.8 / 16.7 and 24.8; 1024x512 30 and 36 / 29 and 43.
-constexpr int kResMinSteps = 2;
+// Fewer steps than this are launched one by one: a resident launch loads and
+// stores the state once more. Two steps pay up to about 400,000 nodes in FP32 and
+// 550,000 in the deviation forms (whose step by launches is slower), and in narrow
+// domains, whose strips are mostly empty in the step kernel. Measured (us for 2
+// and 3 steps, resident / one by one): 128x64 FP32 8.3 and 9.8 / 16.5 and 24.8;
+// 8192x40 FP32 20.6 and 24.8 / 22.6 and 36.9; 1024x512 FP32 27.8 and 33.4 / 24.7
+// and 36.9, FP32 deviations 28.8 and 36.9 / 28.7 and 43.1, FP16 30.7 and 37 / 32.1
+// and 49; 1024x580 FP32 30.8 and 36.9 / 24.6 and 36.9, FP32 deviations 31.7 and
+// 39.0 / 28.7 and 43.1; 90x5000 FP32 24.6 / 36.9 (2 steps).
+int resident_min_steps(const lbm_ctx* c)
+{
+    const long long most = c->prm.storage == LBM_FP32 ? 400000 : 550000;
+    return (long long)c->g.nx * c->g.ny > most && c->g.nx >= 256 ? 3 : 2;
+}
 
 // The next launch of `left` steps: n of them, with an exchange every k. An even
 // number of steps leaves the state in the buffer where it was, as steps one by
@@ -1473,14 +1483,15 @@ lbm_status lbm_step(lbm_ctx* c, int64_t nsteps)
     if (s) return s;
     if (nsteps < 0) return fail(c, LBM_EINVAL, "nsteps must be >= 0");
     const int K = c->prm.obs_every;
+    const int least = resident_min_steps(c);
     int capture = -1;  // whether the stream is being captured (a captured call keeps its launches), asked once
     for (int64_t k = 0; k < nsteps; ++k) {
         if (c->exch && capture != 1) {
-            // plain steps up to the next observed one: on the chip from
-            // kResMinSteps on
+            // plain steps up to the next observed one: on the chip if there
+            // are enough of them
             const int64_t run = K == 0 ? nsteps - k : (c->t % K == 0 ? 0 : std::min<int64_t>(nsteps - k, K - c->t % K));
-            if (run >= kResMinSteps && capture < 0) capture = capturing(c->stream) ? 1 : 0;
-            if (run >= kResMinSteps && capture == 0) {
+            if (run >= least && capture < 0) capture = capturing(c->stream) ? 1 : 0;
+            if (run >= least && capture == 0) {
                 bool done;
                 const int64_t t0 = c->t;
                 if ((s = resident_steps(c, run, &done))) return s;

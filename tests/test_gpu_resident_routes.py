@@ -48,6 +48,18 @@ def test_other_calls_are_not(lbm, more):
     assert lat.resident_launches == 0
 
 
+@pytest.mark.parametrize("nx,ny,storage,two", [
+    (128, 64, 0, 1), (1024, 290, 0, 1), (90, 5000, 0, 1), (1024, 512, 0, 0), (2048, 256, 0, 0), (1024, 512, 1, 1),
+    (1024, 580, 1, 0), (1024, 512, 2, 1),
+])
+def test_two_steps_of_large_domains_are_not(lbm, nx, ny, storage, two):
+    lat = ready(lbm, nx, ny, storage=storage)
+    lat.step(2)
+    assert lat.resident_launches == two
+    lat.step(3)
+    assert lat.resident_launches == two + 1
+
+
 def test_captured_steps_are_not(lbm):
     import torch
     st = torch.cuda.Stream()
