@@ -1073,11 +1073,18 @@ bool capturing(cudaStream_t st)
     return cs != cudaStreamCaptureStatusNone;
 }
 
-// Steps per resident launch at most: about a millisecond or two, so that
-// other streams' work gets its turn. Even, so that only a call's last launch
-// can have an odd number of steps.
-constexpr int kResChunk = 1024;
-static_assert(kResChunk % 2 == 0, "an even number of steps returns the state to its buffer");
+// Steps per resident launch at most: about three milliseconds by the plan's
+// estimate (the launch holds all its SMs), so that other streams' work gets its
+// turn. Even, so that only a call's last launch can have an odd number of steps.
+// Each launch more costs about 15 us (1000 steps of 1024x128 in two launches: 2877
+// us against 2860 in one).
+constexpr double kResLaunchUs = 3000.0;
+constexpr double kResClock = 1900.0;  // SM cycles per us
+int resident_chunk(const ResPlan& r)
+{
+    return std::max(8, int(std::min(1024.0, kResLaunchUs * kResClock / r.cycles)) / 2 * 2);
+}
+
 // Fewer steps than this are launched one by one: a resident launch loads and
 // stores the state once more. Two steps pay up to about 400,000 nodes in FP32 and
 // 550,000 in the deviation forms (whose step by launches is slower), and in narrow
@@ -1101,11 +1108,11 @@ struct ResLaunch {
     int n, k;
     bool swap;
 };
-ResLaunch resident_launch(int64_t left, int k)
+ResLaunch resident_launch(int64_t left, const ResPlan& r)
 {
-    const int n = int(std::min<int64_t>(left, kResChunk));
+    const int n = int(std::min<int64_t>(left, resident_chunk(r)));
     const bool swap = n % 2 != 0;
-    return {n, swap || n > k ? k : n / 2, swap};
+    return {n, swap || n > r.k ? r.k : n / 2, swap};
 }
 
 // nsteps plain steps of a domain that fits on the chip. *done = false if this
@@ -1116,7 +1123,7 @@ lbm_status resident_steps(lbm_ctx* c, int64_t nsteps, bool* done)
     const void* fn = resident_fn(c->prm.storage, c->ph.tau == 1.f, r.j, false);
     *done = true;
     while (nsteps > 0) {
-        ResLaunch l = resident_launch(nsteps, r.k);
+        ResLaunch l = resident_launch(nsteps, r);
         const float* in = c->cur;
         float* out = l.swap ? c->nxt : c->cur;
         int tx = r.tx, ty = r.ty, cap = r.edge_cap, stride = int(c->L.exch_bytes / 2 / sizeof(uint4));
@@ -2114,7 +2121,7 @@ void plan_groups(lbm_batch* b)
         }
         b->groups.push_back(gr);
     }
-    b->res_us = best / 1900.0;  // at 1.9 GHz
+    b->res_us = best / kResClock;
     // a launch, and the state in and out once
     b->res_us_once = 8.0 * double(b->groups.size()) + double(nodes) * 72.0 / 4e6;
 }
@@ -2144,7 +2151,7 @@ lbm_status resident_batch_steps(lbm_batch* b, int64_t nsteps, bool* done)
         const int2* ctas = b->d_ctas + gr.first;
         int cap = gr.plan.edge_cap, stride = gr.ctas * res_records(b->storage) * cap;
         for (int64_t left = nsteps; left > 0;) {
-            ResLaunch l = resident_launch(left, gr.plan.k);
+            ResLaunch l = resident_launch(left, gr.plan);
             int in = 0, out = l.swap ? 1 : 0;  // (a swapping launch is the last)
             uint32_t tag = 0;
             if ((s = take_tags(&b->res_tag, l.n, b->exch, b->exch_bytes, b->stream, &tag)))

@@ -99,3 +99,34 @@ def test_larger_plans_stay_resident(lbm):
         lat.step(20)
         lat.observables()
         assert lat.resident_launches == 1
+
+
+@pytest.mark.parametrize("nx,ny,storage", [(128, 64, 0), (1024, 128, 1), (1024, 512, 0), (2048, 256, 1), (1024, 580, 2)])
+def test_a_launch_holds_the_gpu_for_some_milliseconds(lbm, nx, ny, storage):
+    """Three by the plan's estimate, which may be off by half."""
+    import torch
+    lat = ready(lbm, nx, ny, storage=storage)
+    lat.step(1024)
+    before, start, end = lat.resident_launches, *(torch.cuda.Event(enable_timing=True) for _ in range(2))
+    start.record()
+    lat.step(2048)
+    end.record()
+    torch.cuda.synchronize()
+    assert start.elapsed_time(end) / (lat.resident_launches - before) < 4.5
+
+
+def test_a_group_holds_the_gpu_for_some_milliseconds(lbm):
+    import torch
+    p = dict(wl.PAPER, storage=lbm.LBM_FP32_DEV)
+    b = lbm.Batch([dict(nx=256, ny=64, **p) for _ in range(64)])
+    for d in b.domains:
+        mask, _ = domain(256, 64, True, 1)
+        d.set_geometry(mask)
+        d.set_rho(np.where(mask, 0.0, 1.5))
+    b.step(500)
+    before, start, end = b.resident_launches, *(torch.cuda.Event(enable_timing=True) for _ in range(2))
+    start.record()
+    b.step(1000)
+    end.record()
+    torch.cuda.synchronize()
+    assert start.elapsed_time(end) / (b.resident_launches - before) < 4.5
