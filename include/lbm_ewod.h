@@ -294,6 +294,20 @@ lbm_ctx *lbm_batch_domain(lbm_batch *b, int32_t i);
  * covering all active domains; pairs of steps run as one CUDA graph. */
 lbm_status lbm_batch_step(lbm_batch *b, int64_t nsteps);
 
+/* How count domains would be grouped to run on the chip (host arithmetic only, no
+ * GPU needed): out[0 .. n-1] (may be NULL with n = 0) gets the first n groups.
+ * Each group is one launch of `ctas` CTAs of `threads` threads and `smem` bytes;
+ * every `interval` steps a CTA publishes up to `edge_nodes` nodes. edge_nodes
+ * bounds the published nodes of a group (0: what a batch's workspace holds).
+ * Returns the number of groups, 0 where some domain does not fit on the chip or
+ * has a forced layout or tile height, -1 for invalid arguments. */
+typedef struct {
+    int32_t domains, ctas, threads, interval, edge_nodes, smem;
+    double cycles; /* estimated SM cycles per step */
+} lbm_resident_group;
+int32_t lbm_batch_resident_plan(const lbm_params *params, int32_t count, int64_t edge_nodes,
+                                lbm_resident_group *out, int32_t n);
+
 /* Launches of the resident kernel for this batch so far, and the groups (one
  * launch each) of the last resident call's domains; -1 for NULL. */
 int64_t lbm_batch_resident_launches(const lbm_batch *b);

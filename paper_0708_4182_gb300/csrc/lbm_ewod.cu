@@ -132,6 +132,9 @@ bool res_try(int storage, bool t1, int w, int h, int k, int per_sm, ResPlan* r)
     return r->cycles >= 0.0;
 }
 
+// Resident steps take no forced thread layout or tile height.
+bool res_automatic(const lbm_params& p) { return p.layout == LBM_LAYOUT_AUTO && p.tile_rows == 0; }
+
 // The tiling with the fewest estimated cycles per step.
 ResPlan res_plan(int nx, int ny, int storage, bool t1)
 {
@@ -179,7 +182,7 @@ Layout layout_of(const lbm_params* p, bool single)
     if (L.staging_bytes < size_t(9) * p->nx * sizeof(double)) L.staging_bytes = size_t(9) * p->nx * sizeof(double);
     L.off_staging = o; o = align_up(o + L.staging_bytes, 256);
     L.off_exch = o;
-    if (single && p->layout == LBM_LAYOUT_AUTO && p->tile_rows == 0) {
+    if (single && res_automatic(*p)) {
         L.res = res_plan(p->nx, p->ny, p->storage, float(p->tau) == 1.f);
         L.exch_bytes = size_t(2) * L.res.tiles() * res_records(p->storage) * L.res.edge_cap * sizeof(uint4);
     }
@@ -1758,6 +1761,20 @@ const char* lbm_noalloc_last_error(void) { return g_noalloc_err; }
 // ===========================================================================
 // Batches: many domains of different sizes stepped by one launch per step.
 
+namespace {
+
+// The active domains of a batch in groups that fit on the chip, each one launch
+// of CTAs first .. first + ctas - 1 of the CTA table.
+struct ResGroup { ResPlan plan; int first, ctas, domains; };
+struct ResGroups {
+    std::vector<ResGroup> groups;
+    std::vector<int4> shape;  // per domain: tx, ty, first CTA of its group's launch
+    std::vector<int2> ctas;   // (domain, tile) of every CTA
+    double step_us = 0.0, once_us = 0.0, walk_us = 0.0;  // estimated time per step, per call; of the tile walk per step
+};
+
+}  // namespace
+
 struct lbm_batch {
     int count = 0;
     int storage = 0;
@@ -1790,21 +1807,15 @@ struct lbm_batch {
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
     int graph_ntiles = -1, graph_grid = -1;
-    // resident steps: the active domains in groups that fit on the chip, each
-    // one launch of CTAs first .. first + ctas - 1 of the CTA table
-    struct Group { ResPlan plan; int first, ctas; };
-    bool res_allowed = false;            // automatic layout and tiling throughout
-    std::vector<Group> groups;
-    double res_us = 0.0, res_us_once = 0.0, walk_us = 0.0;  // estimated time per step, per call; of the tile walk per step
+    bool res_allowed = false;            // resident steps: automatic layout and tiling throughout
+    ResGroups res;
     bool groups_dirty = true;
     uint4* exch = nullptr;
     size_t exch_bytes = 0;
     uint32_t res_tag = 1;
     int64_t res_launches = 0;
-    int4* d_shape = nullptr;             // per domain: tx, ty, first CTA of its group's launch
-    int2* d_ctas = nullptr;              // (domain, tile) of every CTA
-    std::vector<int4> h_shape;
-    std::vector<int2> h_ctas;
+    int4* d_shape = nullptr;             // res.shape and res.ctas on the device
+    int2* d_ctas = nullptr;
     char err[512] = {0};
 };
 
@@ -2032,25 +2043,25 @@ lbm_status batch_graph(lbm_batch* b)
 
 // Group the active domains for resident steps (largest first into the first
 // group with room), for the tile height and exchange interval whose groups
-// take the fewest estimated cycles together. groups stays empty where a
-// domain does not fit on the chip.
-void plan_groups(lbm_batch* b)
+// take the fewest estimated cycles together. A group's CTAs publish edge_nodes
+// nodes at most. groups stays empty where a domain does not fit on the chip.
+ResGroups plan_groups(const std::vector<int2>& size, const std::vector<unsigned char>& active, int storage, bool tau1,
+                      long long edge_nodes)
 {
-    b->groups.clear();
-    b->groups_dirty = false;
+    ResGroups out;
+    out.shape.resize(size.size());
     std::vector<int> order;
     long long nodes = 0;
-    for (int d = 0; d < b->count; ++d)
-        if (b->active[d]) {
+    auto area = [&](int d) { return (long long)size[d].x * size[d].y; };
+    for (int d = 0; d < int(size.size()); ++d)
+        if (active[d]) {
             order.push_back(d);
-            nodes += (long long)b->ctx[d]->g.nx * b->ctx[d]->g.ny;
+            nodes += area(d);
         }
-    std::sort(order.begin(), order.end(), [&](int x, int y) {
-        return (long long)b->ctx[x]->g.nx * b->ctx[x]->g.ny > (long long)b->ctx[y]->g.nx * b->ctx[y]->g.ny;
-    });
+    std::sort(order.begin(), order.end(), [&](int x, int y) { return area(x) > area(y); });
     // the tile walk: about 12 us of latency and 80 GLUPS (measured: 64 channels
     // of 256x64 28 us, 256 uneven channels 81.7 GLUPS in FP32)
-    b->walk_us = 12.0 + double(nodes) / 80e3;
+    out.walk_us = 12.0 + double(nodes) / 80e3;
     struct Trial { int w = 0, h = 0, ctas = 0, edge = 0, hmax = 0; std::vector<int> doms; };
     static const int heights[] = {4, 8, 12, 16, 20, 24, 28, 32, 40, 48, 56, 64, 72, 80, 96, 112, 128, 144};
     double best = -1.0;
@@ -2062,20 +2073,25 @@ void plan_groups(lbm_batch* b)
             // CTAs of this height that fit on an SM
             ResPlan r;
             int per_sm = 0;
-            while (per_sm < 4 && res_try(b->storage, b->tau1, wmax, hmax, k, per_sm + 1, &r)) ++per_sm;
+            while (per_sm < 4 && res_try(storage, tau1, wmax, hmax, k, per_sm + 1, &r)) ++per_sm;
             if (!per_sm) continue;
             std::vector<Trial> trial;
             bool ok = true;
             for (int d : order) {
-                const Geom& g = b->ctx[d]->g;
-                const int tx = (g.nx + wmax - 1) / wmax, ty = (g.ny + hmax - 1) / hmax;
-                const int w = (g.nx + tx - 1) / tx, h = (g.ny + ty - 1) / ty;
+                const int2 g = size[d];
+                const int tx = (g.x + wmax - 1) / wmax, ty = (g.y + hmax - 1) / hmax;
+                const int w = (g.x + tx - 1) / tx, h = (g.y + ty - 1) / ty;
                 const int edge = res_edge_nodes(w, h, 2 * k);
-                if (tx * ty > per_sm * kResSms) { ok = false; break; }
+                // whether a group of `ctas` CTAs and tiles of up to `most` edge
+                // nodes has room for this domain (an empty one too: a domain
+                // that opens a group is bound by the same limits)
+                auto room = [&](int ctas, int most) {
+                    return (long long)ctas + (long long)tx * ty <= per_sm * kResSms &&
+                           ((long long)ctas + tx * ty) * std::max(most, edge) <= edge_nodes;
+                };
+                if (!room(0, 0)) { ok = false; break; }
                 size_t i = 0;
-                while (i < trial.size() && (trial[i].ctas + tx * ty > per_sm * kResSms ||
-                                            (trial[i].ctas + tx * ty) * std::max(trial[i].edge, edge) > kResEdgeNodes))
-                    ++i;
+                while (i < trial.size() && !room(trial[i].ctas, trial[i].edge)) ++i;
                 if (i == trial.size()) trial.emplace_back();
                 Trial& t = trial[i];
                 t.ctas += tx * ty;
@@ -2089,7 +2105,7 @@ void plan_groups(lbm_batch* b)
             double cost = 0.0;
             std::vector<ResPlan> rs;
             for (const Trial& t : trial) {
-                if (!res_try(b->storage, b->tau1, t.w, t.h, k, (t.ctas + kResSms - 1) / kResSms, &r)) { ok = false; break; }
+                if (!res_try(storage, tau1, t.w, t.h, k, (t.ctas + kResSms - 1) / kResSms, &r)) { ok = false; break; }
                 r.edge_cap = t.edge;
                 cost += r.cycles;
                 rs.push_back(r);
@@ -2101,29 +2117,36 @@ void plan_groups(lbm_batch* b)
             }
         }
     }
-    if (best < 0.0) return;
-    b->h_ctas.clear();
+    if (best < 0.0) return out;
     for (size_t i = 0; i < pick.size(); ++i) {
-        lbm_batch::Group gr{plans[i], int(b->h_ctas.size()), pick[i].ctas};
-        int first = 0;
+        const int first = int(out.ctas.size()), wmax = kResP - 4 * plans[i].k;
         for (int d : pick[i].doms) {
-            const Geom& g = b->ctx[d]->g;
-            const int wmax = kResP - 4 * gr.plan.k;
-            const int tx = (g.nx + wmax - 1) / wmax, ty = (g.ny + pick[i].hmax - 1) / pick[i].hmax;
-            b->h_shape[d] = make_int4(tx, ty, first, 0);
-            for (int t = 0; t < tx * ty; ++t) b->h_ctas.push_back(make_int2(d, t));
-            first += tx * ty;
+            const int tx = (size[d].x + wmax - 1) / wmax, ty = (size[d].y + pick[i].hmax - 1) / pick[i].hmax;
+            out.shape[d] = make_int4(tx, ty, int(out.ctas.size()) - first, 0);
+            for (int t = 0; t < tx * ty; ++t) out.ctas.push_back(make_int2(d, t));
         }
-        gr.ctas = first;
-        if (!resident_fits(resident_fn(b->storage, b->tau1, gr.plan.j, true), gr.plan, gr.ctas, b->sm_count)) {
-            b->groups.clear();
+        out.groups.push_back({plans[i], first, int(out.ctas.size()) - first, int(pick[i].doms.size())});
+    }
+    out.step_us = best / kResClock;
+    // a launch, and the state in and out once
+    out.once_us = 8.0 * double(out.groups.size()) + double(nodes) * 72.0 / 4e6;
+    return out;
+}
+
+// The groups of the batch's active domains; none where a group's CTAs would not
+// be resident together on this device, or its records would not fit.
+void group_batch(lbm_batch* b)
+{
+    b->groups_dirty = false;
+    std::vector<int2> size(b->count);
+    for (int d = 0; d < b->count; ++d) size[d] = make_int2(b->ctx[d]->g.nx, b->ctx[d]->g.ny);
+    b->res = plan_groups(size, b->active, b->storage, b->tau1, kResEdgeNodes);
+    for (const ResGroup& g : b->res.groups)
+        if (size_t(2) * res_records(b->storage) * g.ctas * g.plan.edge_cap * sizeof(uint4) > b->exch_bytes ||
+            !resident_fits(resident_fn(b->storage, b->tau1, g.plan.j, true), g.plan, g.ctas, b->sm_count)) {
+            b->res.groups.clear();
             return;
         }
-        b->groups.push_back(gr);
-    }
-    b->res_us = best / kResClock;
-    // a launch, and the state in and out once
-    b->res_us_once = 8.0 * double(b->groups.size()) + double(nodes) * 72.0 / 4e6;
 }
 
 // nsteps plain steps of the active domains, group after group. *done = false
@@ -2134,19 +2157,20 @@ lbm_status resident_batch_steps(lbm_batch* b, int64_t nsteps, bool* done)
     if (!b->res_allowed || capturing(b->stream)) return LBM_OK;
     lbm_status s;
     if (b->groups_dirty) {
-        plan_groups(b);
-        if (!b->groups.empty()) {
-            if ((s = bcheck(b, cudaMemcpyAsync(b->d_shape, b->h_shape.data(), b->count * sizeof(int4),
+        group_batch(b);
+        if (!b->res.groups.empty()) {
+            if ((s = bcheck(b, cudaMemcpyAsync(b->d_shape, b->res.shape.data(), b->count * sizeof(int4),
                                                cudaMemcpyHostToDevice, b->stream), "tiling upload")) ||
-                (s = bcheck(b, cudaMemcpyAsync(b->d_ctas, b->h_ctas.data(), b->h_ctas.size() * sizeof(int2),
+                (s = bcheck(b, cudaMemcpyAsync(b->d_ctas, b->res.ctas.data(), b->res.ctas.size() * sizeof(int2),
                                                cudaMemcpyHostToDevice, b->stream), "CTA table upload")))
                 return s;
         }
     }
     // by a clear margin: for large sweeps the two are within the estimates' error
     // (64 uneven channels, 11.7 M nodes: 11.6 ms resident, 11.4 ms by the walk)
-    if (b->groups.empty() || 1.3 * (b->res_us * double(nsteps) + b->res_us_once) >= b->walk_us * double(nsteps)) return LBM_OK;
-    for (const lbm_batch::Group& gr : b->groups) {
+    const ResGroups& res = b->res;
+    if (res.groups.empty() || 1.3 * (res.step_us * double(nsteps) + res.once_us) >= res.walk_us * double(nsteps)) return LBM_OK;
+    for (const ResGroup& gr : res.groups) {
         const void* fn = resident_fn(b->storage, b->tau1, gr.plan.j, true);
         const int2* ctas = b->d_ctas + gr.first;
         int cap = gr.plan.edge_cap, stride = gr.ctas * res_records(b->storage) * cap;
@@ -2158,7 +2182,7 @@ lbm_status resident_batch_steps(lbm_batch* b, int64_t nsteps, bool* done)
                 return bfail(b, s, "exchange buffer clear");
             void* args[] = {&b->d_dom, &b->d_shape, &ctas, &in, &out, &l.k, &b->exch, &stride, &cap, &tag, &l.n, &b->d_status};
             const cudaError_t e = cudaLaunchCooperativeKernel(fn, dim3(gr.ctas), dim3(gr.plan.nt), args, gr.plan.smem, b->stream);
-            if (e == cudaErrorCooperativeLaunchTooLarge && left == nsteps && &gr == &b->groups.front()) {
+            if (e == cudaErrorCooperativeLaunchTooLarge && left == nsteps && &gr == &res.groups.front()) {
                 cudaGetLastError();
                 b->res_allowed = false;
                 return LBM_OK;
@@ -2239,6 +2263,29 @@ lbm_status batch_observe(lbm_batch* b, const std::vector<unsigned char>& want, l
 
 extern "C" {
 
+int32_t lbm_batch_resident_plan(const lbm_params* params, int32_t count, int64_t edge_nodes, lbm_resident_group* out,
+                                int32_t n)
+{
+    const char* why;
+    if (!params || count < 1 || edge_nodes < 0 || n < 0 || (n > 0 && !out)) return -1;
+    std::vector<int2> size(count);
+    bool automatic = true, tau1 = true;
+    for (int d = 0; d < count; ++d) {
+        if (!params_valid(&params[d], &why) || params[d].storage != params[0].storage) return -1;
+        size[d] = make_int2(params[d].nx, params[d].ny);
+        automatic = automatic && res_automatic(params[d]);
+        tau1 = tau1 && float(params[d].tau) == 1.f;
+    }
+    if (!automatic) return 0;
+    const ResGroups r = plan_groups(size, std::vector<unsigned char>(count, 1), params[0].storage, tau1,
+                                    edge_nodes ? edge_nodes : kResEdgeNodes);
+    for (int i = 0; i < n && i < int(r.groups.size()); ++i) {
+        const ResGroup& g = r.groups[i];
+        out[i] = {g.domains, g.ctas, g.plan.nt, g.plan.k, g.plan.edge_cap, int32_t(g.plan.smem), g.plan.cycles};
+    }
+    return int32_t(r.groups.size());
+}
+
 size_t lbm_batch_workspace_bytes(const lbm_params* params, int32_t count)
 {
     BatchLayout L;
@@ -2290,10 +2337,9 @@ lbm_status lbm_batch_create(const lbm_params* params, int32_t count, void* d_wor
     b->d_ctas = reinterpret_cast<int2*>(ws + L.off_ctas);
     b->exch = reinterpret_cast<uint4*>(ws + L.off_exch);
     b->exch_bytes = L.exch_bytes;
-    b->h_shape.resize(count);
     b->res_allowed = true;
     for (int d = 0; d < count; ++d)
-        if (params[d].layout != LBM_LAYOUT_AUTO || params[d].tile_rows != 0) b->res_allowed = false;
+        if (!res_automatic(params[d])) b->res_allowed = false;
     cudaError_t e = cudaMemsetAsync(b->exch, 0, b->exch_bytes, b->stream);
     for (int d = 0; d < count; ++d)
         if (b->ctx[d]->ph.tau != 1.f) b->tau1 = false;
@@ -2392,7 +2438,7 @@ lbm_status lbm_batch_step(lbm_batch* b, int64_t nsteps)
 
 int64_t lbm_batch_resident_launches(const lbm_batch* b) { return b ? b->res_launches : -1; }
 
-int32_t lbm_batch_resident_groups(const lbm_batch* b) { return b ? int32_t(b->groups.size()) : -1; }
+int32_t lbm_batch_resident_groups(const lbm_batch* b) { return b ? int32_t(b->res.groups.size()) : -1; }
 
 lbm_status lbm_batch_observables(lbm_batch* b, lbm_obs* out)
 {

@@ -434,6 +434,8 @@ def _batch_lib():
             "lbm_batch_create": (ctypes.c_int, [P, ctypes.c_int32, vp, ctypes.c_size_t, vp, ctypes.POINTER(vp)]),
             "lbm_batch_domain": (vp, [vp, ctypes.c_int32]),
             "lbm_batch_step": (ctypes.c_int, [vp, ctypes.c_int64]),
+            "lbm_batch_resident_plan": (ctypes.c_int32, [P, ctypes.c_int32, ctypes.c_int64,
+                                                         ctypes.POINTER(lbm_resident_group), ctypes.c_int32]),
             "lbm_batch_resident_launches": (ctypes.c_int64, [vp]),
             "lbm_batch_resident_groups": (ctypes.c_int32, [vp]),
             "lbm_batch_observables": (ctypes.c_int, [vp, O]),
@@ -460,6 +462,22 @@ def _batch_lib():
             fn.restype, fn.argtypes = res, args
         lib._batch_sigs = True
     return lib
+
+
+class lbm_resident_group(ctypes.Structure):
+    _fields_ = [(k, ctypes.c_int32) for k in ("domains", "ctas", "threads", "interval", "edge_nodes", "smem")] + \
+        [("cycles", ctypes.c_double)]
+
+
+def lbm_batch_resident_plan(specs, edge_nodes: int = 0) -> list:
+    """How the domains of ``specs`` (as for ``Batch``) would be grouped to run on
+    the chip: one dict per group, none where they would not. No GPU needed."""
+    arr = (lbm_params * len(specs))(*[make_params(**sp) for sp in specs])
+    out = (lbm_resident_group * len(specs))()
+    n = _batch_lib().lbm_batch_resident_plan(arr, len(specs), int(edge_nodes), out, len(specs))
+    if n < 0:
+        raise LbmError(LBM_EINVAL, "invalid batch parameters")
+    return [{k: getattr(g, k) for k, _ in g._fields_} for g in out[:n]]
 
 
 class Batch:
