@@ -1845,6 +1845,7 @@ struct BatchLayout {
     std::vector<size_t> off;  // per-domain workspace offsets
     size_t off_dom, off_tiles, off_status, off_rec, off_ptrs, off_nctas, off_invnx, off_step, off_want, total;
     size_t off_shape, off_ctas, off_exch, exch_bytes;
+    bool automatic;  // no forced layout or tile height
     int max_tiles;
 };
 
@@ -1871,8 +1872,10 @@ bool batch_layout(const lbm_params* p, int count, BatchLayout* L, const char** w
     L->off_step = o; o = align_up(o + count * sizeof(long long), 256);
     L->off_want = o; o = align_up(o + count, 256);
     L->off_shape = o; o = align_up(o + count * sizeof(int4), 256);
-    L->off_ctas = o; o = align_up(o + size_t(count) * kResCtas * sizeof(int2), 256);
-    L->exch_bytes = size_t(2) * res_records(p[0].storage) * kResEdgeNodes * sizeof(uint4);
+    // the CTA table and the exchange records, where resident steps are possible
+    L->automatic = std::all_of(p, p + count, res_automatic);
+    L->off_ctas = o; o = align_up(o + (L->automatic ? size_t(count) * kResCtas * sizeof(int2) : 0), 256);
+    L->exch_bytes = L->automatic ? size_t(2) * res_records(p[0].storage) * kResEdgeNodes * sizeof(uint4) : 0;
     L->off_exch = o; o = align_up(o + L->exch_bytes, 256);
     L->total = o;
     return true;
@@ -2337,10 +2340,8 @@ lbm_status lbm_batch_create(const lbm_params* params, int32_t count, void* d_wor
     b->d_ctas = reinterpret_cast<int2*>(ws + L.off_ctas);
     b->exch = reinterpret_cast<uint4*>(ws + L.off_exch);
     b->exch_bytes = L.exch_bytes;
-    b->res_allowed = true;
-    for (int d = 0; d < count; ++d)
-        if (!res_automatic(params[d])) b->res_allowed = false;
-    cudaError_t e = cudaMemsetAsync(b->exch, 0, b->exch_bytes, b->stream);
+    b->res_allowed = L.automatic;
+    cudaError_t e = L.automatic ? cudaMemsetAsync(b->exch, 0, b->exch_bytes, b->stream) : cudaSuccess;
     for (int d = 0; d < count; ++d)
         if (b->ctx[d]->ph.tau != 1.f) b->tau1 = false;
     // Thread layout (32-bit forms), by the rule of a single domain applied to

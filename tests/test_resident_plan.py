@@ -57,3 +57,18 @@ def test_forced_layouts_are_not_grouped(lbm):
         lbm.lbm_batch_resident_plan([dict(nx=0, ny=5)])
     with pytest.raises(lbm.LbmError):
         lbm.lbm_batch_resident_plan([dict(nx=64, ny=5), dict(nx=64, ny=5, storage=1)])
+
+
+@pytest.mark.parametrize("storage", [0, 3])
+def test_workspace_without_resident_steps(lbm, storage):
+    """A batch with a forced layout or height carries no exchange buffer (16 bytes
+    per record, two buffers of 2^18 nodes) and no CTA table."""
+    sp = [dict(nx=256, ny=64, storage=storage), dict(nx=40, ny=30, storage=storage)]
+
+    def size(**more):
+        arr = (lbm.lbm_params * 2)(*[lbm.make_params(**{**sp[0], **more}), lbm.make_params(**sp[1])])
+        return lbm._batch_lib().lbm_batch_workspace_bytes(arr, 2)
+
+    exchange = 2 * 16 * STORAGE_RECORDS[storage] << 18
+    for more in (dict(layout=1), dict(layout=2), dict(tile_rows=8)):
+        assert size() - size(**more) >= exchange
