@@ -214,12 +214,14 @@ lbm_status lbm_step(lbm_ctx *ctx, int64_t nsteps);
  * way lbm_step went, for tests and tuning. */
 int64_t lbm_resident_launches(const lbm_ctx *ctx);
 
-/* Self-test of the device-side timeout path (no counterpart in the paper):
+/* Self-test of the device-side timeout paths (no counterpart in the paper):
  * one kernel waits, with the step kernel's bounded mbarrier wait (2^18
- * polls), on an mbarrier phase that nothing completes. The wait gives up and
- * raises the context's error flag, and the call returns LBM_ETIMEOUT once the
- * stream has drained (about a second). The flag is cleared when read, so the
- * context stays usable. Any other status means the timeout path is broken. */
+ * polls), on an mbarrier phase that nothing completes, then one polls, with
+ * the resident steps' bounded wait (2^20 polls), records that nothing writes.
+ * Each wait gives up and raises the context's error flag, and the call returns
+ * LBM_ETIMEOUT once the stream has drained (about two seconds). The flag is
+ * cleared when read, so the context stays usable. Any other status means a
+ * timeout path is broken. */
 lbm_status lbm_selftest_timeout(lbm_ctx *ctx);
 
 /* Observables of the current state (Eq. 11 and mass/momentum bookkeeping),

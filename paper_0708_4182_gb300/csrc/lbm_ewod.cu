@@ -560,6 +560,15 @@ __global__ void wait_selftest_kernel(int* err)
     }
 }
 
+// The same for the resident steps' wait: records that nothing writes. The second
+// poll does not wait any more.
+__global__ void record_selftest_kernel(const uint4* records, uint32_t tag, int* err)
+{
+    uint4 r[1];
+    bool alive = true;
+    for (int k = 0; k < 2; ++k) get_node_records(records + threadIdx.x, 1, tag, err, alive, r);
+}
+
 // Mean velocity profile across the channel: out[y] = (1/nx) sum_x u_x(x, y)
 // from a kFields array (solid nodes hold 0), one block per row, FP64 tree sum.
 __global__ void ux_profile_kernel(const double* __restrict__ fields, Geom g, double* __restrict__ out)
@@ -1551,11 +1560,22 @@ static lbm_status read_record(lbm_ctx* c, const lbm_obs* rec, lbm_obs* out)
 lbm_status lbm_selftest_timeout(lbm_ctx* c)
 {
     if (!c) return LBM_EINVAL;
-    wait_selftest_kernel<<<1, 32, 0, c->stream>>>(c->status);
-    lbm_status s = check_launch(c, "self-test kernel launch");
-    if (s) return s;
-    if ((s = check_cuda(c, cudaStreamSynchronize(c->stream), "self-test sync"))) return s;
-    return check_status(c);
+    // first the step kernel's wait, then the resident steps' (on two zeroed
+    // records of the staging buffer, which holds nothing between calls)
+    lbm_status s;
+    for (int k = 0; k < 2; ++k) {
+        if (k == 0) {
+            wait_selftest_kernel<<<1, 32, 0, c->stream>>>(c->status);
+        } else {
+            if ((s = check_cuda(c, cudaMemsetAsync(c->staging, 0, 2 * sizeof(uint4), c->stream), "self-test clear"))) return s;
+            record_selftest_kernel<<<1, 2, 0, c->stream>>>(reinterpret_cast<const uint4*>(c->staging), 1, c->status);
+        }
+        if ((s = check_launch(c, "self-test kernel launch"))) return s;
+        if ((s = check_cuda(c, cudaStreamSynchronize(c->stream), "self-test sync"))) return s;
+        s = check_status(c);
+        if (s != LBM_ETIMEOUT) return s;
+    }
+    return s;
 }
 
 lbm_status lbm_observables(lbm_ctx* c, lbm_obs* out)

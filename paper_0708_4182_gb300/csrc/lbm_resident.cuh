@@ -236,6 +236,29 @@ __device__ __forceinline__ void res_pull(const float* __restrict__ m, const floa
 
 constexpr uint32_t kResWaitLimit = 1u << 20;  // polls of a record before giving up (about a second)
 
+// Poll a published node's records (stride apart) until all carry the tag. A
+// thread that gives up raises the error flag and from then on (alive = false)
+// takes what it finds.
+template <int NB>
+__device__ __forceinline__ void get_node_records(const uint4* q, int stride, uint32_t tag, int* err, bool& alive,
+                                                 uint4 (&r)[NB])
+{
+    bool ok = false;
+    for (uint32_t i = 0; i < kResWaitLimit; ++i) {
+        ok = true;
+#pragma unroll
+        for (int b = 0; b < NB; ++b) {
+            r[b] = get_record(q + b * stride);
+            ok = ok && r[b].w == tag;
+        }
+        if (ok || !alive) break;
+    }
+    if (!ok && alive) {
+        atomicOr(err, 1);
+        alive = false;
+    }
+}
+
 // A node's stored state as 32-bit words: 9 populations, rho* and 8
 // deviations, or rho* and 4 pairs of 16-bit deviations.
 template <int ST> constexpr int kResWords = is16(ST) ? 5 : 9;
@@ -449,20 +472,7 @@ __device__ __forceinline__ void run_resident(const Geom& g, const Phys& p, const
             const int2 hk = halo[k];
             const uint4* q = ex + hk.x;
             uint4 r[NB];
-            bool ok = false;
-            for (uint32_t i = 0; i < kResWaitLimit; ++i) {
-                ok = true;
-#pragma unroll
-                for (int b = 0; b < NB; ++b) {
-                    r[b] = get_record(q + b * edge_cap);
-                    ok = ok && r[b].w == tag;
-                }
-                if (ok || !alive) break;
-            }
-            if (!ok && alive) {
-                atomicOr(err, 1);
-                alive = false;
-            }
+            get_node_records(q, edge_cap, tag, err, alive, r);
             uint32_t v[NW];
             if constexpr (is16(ST)) {
                 v[0] = r[0].x; v[1] = r[0].y; v[2] = r[0].z; v[3] = r[NB - 1].x; v[4] = r[NB - 1].y;
