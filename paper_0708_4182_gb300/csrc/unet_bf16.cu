@@ -238,7 +238,7 @@ __host__ __device__ constexpr int conv_ntile(int n) { return n % 128 == 0 ? 128 
 // x: NHWC view (channels per pixel ct_in, K = 16 kc channels used), y: NHWC
 // view (ct_out per pixel), wt: packed weights (conv_pack_kernel).
 //
-// The image (or a strip of S of its columns) is taken with one halo column on
+// The image (or a strip of S of its columns, conv_strip) is taken with one halo column on
 // each side, pitch = S + 2 pixels a row, and its padded pixels are numbered row
 // by row. A CTA computes MT x 128 consecutive padded pixels (M = 128 a tile) x
 // NT output channels; the results on halo columns are dropped (3% of a 64-wide
@@ -1379,10 +1379,15 @@ int* err_ptr()
     return p;
 }
 
-// columns of a strip: the whole row up to 256 columns, else the largest
-// multiple of 32 up to 256 that divides it
-int conv_strip(int wd)
+// columns of a strip for CTAs of mt tiles. A CTA stages two rows more than its
+// 128 mt pixels, so few tiles go with short rows: 128 columns where they divide
+// the row (one image of 64x256, 32 -> 32 channels, forward 7.2 us, 8.3 on whole
+// rows; 96 -> 32, 8 images, 24 and 35 us). Else, and for 4 tiles (96 -> 32, 16
+// images: 41 us on whole rows, 47 on 128 columns), the whole row up to 256 columns,
+// or the largest multiple of 32 up to 256 that divides it.
+int conv_strip(int wd, int mt)
 {
+    if (mt < 4 && wd % 128 == 0) return 128;
     if (wd <= 256) return wd;
     int s = 256;
     while (wd % s) s -= 32;
@@ -1393,7 +1398,7 @@ template <int NT, int NG, int CK, int MT>
 int launch_conv_mt(const void* x, int ct_in, int kc, const void* wt, const float* bias, void* y, int ct_out, int cout,
                    int n, int h, int wd, int relu, cudaStream_t st)
 {
-    const int S = conv_strip(wd);
+    const int S = conv_strip(wd, MT);
     constexpr int cols = int(tmem_cols(MT * NT * NG));
     // weight slots: what fits beside a second CTA on the SM (or alone, where
     // the accumulators or 4 slots leave no room for one), up to the K loop's uses
@@ -1424,18 +1429,22 @@ int launch_conv_mt(const void* x, int ct_in, int kc, const void* wt, const float
     return status(cudaGetLastError());
 }
 
-// Rows of whole 128-pixel tiles (CK = 1): MT tiles per CTA, the most of 4, 2
-// and 1 that leave two CTAs per SM; more tiles reuse the staged weights and
-// halo rows.
+// CTAs of mt tiles and n_cta output channels each
+long long conv_ctas(int mt, int n_cta, int cout, int n, int h, int wd)
+{
+    const int S = conv_strip(wd, mt);
+    return (long long)(wd / S) * ((h * (S + 2) + 128 * mt - 1) / (128 * mt)) * (cout / n_cta) * n;
+}
+
+// Rows of a multiple of 128 pixels (CK = 1): MT tiles per CTA, the most of 4, 2
+// and 1 that leave two CTAs per SM; more tiles reuse the staged weights and the
+// window's two extra rows.
 template <int NT, int NG>
 int launch_conv_wide(const void* x, int ct_in, int kc, const void* wt, const float* bias, void* y, int ct_out,
                      int cout, int n, int h, int wd, int relu, cudaStream_t st)
 {
     constexpr int N = NT * NG;
-    const int S = conv_strip(wd);
-    auto ctas = [&](int mt) {
-        return (long long)(wd / S) * ((h * (S + 2) + 128 * mt - 1) / (128 * mt)) * (cout / N) * n;
-    };
+    auto ctas = [&](int mt) { return conv_ctas(mt, N, cout, n, h, wd); };
     if (N <= 64 && ctas(4) >= 304)
         return launch_conv_mt<NT, NG, 1, N <= 64 ? 4 : 1>(x, ct_in, kc, wt, bias, y, ct_out, cout, n, h, wd, relu, st);
     if (ctas(2) >= 304) return launch_conv_mt<NT, NG, 1, 2>(x, ct_in, kc, wt, bias, y, ct_out, cout, n, h, wd, relu, st);
@@ -1450,9 +1459,11 @@ int launch_conv(const void* x, int ct_in, int kc, const void* wt, const float* b
     // tiles: 1); the order of the sums, and so the result, depends on it
     if (wd % 128 == 0) {
         // three blocks of 32 or 64 output channels in one MMA: one of N = 32
-        // takes as long as one of N = 96
+        // takes as long as one of N = 96, three of N = 64 twice as long as one of
+        // 192 (unless that leaves half of the SMs without a CTA: 64 -> 192 at
+        // 32x128, one image, 12.3 us with, 10.3 without)
         if constexpr (NT <= 64)
-            if (cout % (3 * NT) == 0)
+            if (cout % (3 * NT) == 0 && (NT == 32 || conv_ctas(1, 3 * NT, cout, n, h, wd) >= 76))
                 return launch_conv_wide<NT, 3>(x, ct_in, kc, wt, bias, y, ct_out, cout, n, h, wd, relu, st);
         return launch_conv_wide<NT, 1>(x, ct_in, kc, wt, bias, y, ct_out, cout, n, h, wd, relu, st);
     }
