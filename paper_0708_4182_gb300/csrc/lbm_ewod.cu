@@ -86,7 +86,7 @@ bool params_valid(const lbm_params* p, const char** why)
 // CTAs across a domain of nx columns (strips of strip_cols(storage) columns)
 int ctas_x(int nx, int storage) { return (nx + strip_cols(storage) - 1) / strip_cols(storage); }
 
-constexpr int kResSms = 152;                     // SMs of a GB300
+constexpr int kResSms = 152;                     // SMs of a GB300 (fewer: plans that do not fit are not used)
 constexpr size_t kResSmemCta = 227 * 1024;       // shared memory of a CTA at most
 constexpr size_t kResSmemSm = 228 * 1024;        // of an SM; a CTA takes 1 KB of it and its static part as well
 
@@ -566,7 +566,11 @@ __global__ void record_selftest_kernel(const uint4* records, uint32_t tag, int* 
 {
     uint4 r[1];
     bool alive = true;
-    for (int k = 0; k < 2; ++k) get_node_records(records + threadIdx.x, 1, tag, err, alive, r);
+    for (int k = 0; k < 2; ++k)
+        if (!poll_records(records + threadIdx.x, 1, tag, alive, r) && alive) {
+            atomicOr(err, 1);
+            alive = false;
+        }
 }
 
 // Mean velocity profile across the channel: out[y] = (1/nx) sum_x u_x(x, y)

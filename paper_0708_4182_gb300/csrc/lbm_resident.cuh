@@ -32,7 +32,10 @@
 // go to the warps in turn, which spreads the slower rows along a wall
 // (1024x512: 6.8 -> 5.9 us against blocks of rows). Two rows in straight line
 // per warp (spills) and pairs of columns per thread (half the warps) were
-// slower: 4.2 -> 5.0 and 4.2 -> 5.0 us at 1024x256.
+// slower: 4.2 -> 5.0 and 4.2 -> 5.0 us at 1024x256. Counters of 64 steps in one
+// launch (128x64, 1024x128 and 1024x512): issue slots 38, 51 and 63% busy, the
+// shared-memory pipe 14, 34 and 39%, bank conflicts 3, 9 and 15% of its
+// wavefronts; the rest is waiting, at barriers first in the smallest domain.
 //
 // Exchange: a published node is NB records of 16 bytes, three (or fewer)
 // values and the round's tag, each stored and loaded as one 128-bit access, so
@@ -236,12 +239,12 @@ __device__ __forceinline__ void res_pull(const float* __restrict__ m, const floa
 
 constexpr uint32_t kResWaitLimit = 1u << 20;  // polls of a record before giving up (about a second)
 
-// Poll a published node's records (stride apart) until all carry the tag. A
-// thread that gives up raises the error flag and from then on (alive = false)
-// takes what it finds.
+// Poll a published node's records (stride apart) until all carry the tag; false
+// after the last poll (the first, for a thread that has given up before). The
+// caller raises the error flag and gives up: with that in here and `alive` by
+// reference, the step loop's code was 1.4% slower (101 steps of 301x67).
 template <int NB>
-__device__ __forceinline__ void get_node_records(const uint4* q, int stride, uint32_t tag, int* err, bool& alive,
-                                                 uint4 (&r)[NB])
+__device__ __forceinline__ bool poll_records(const uint4* q, int stride, uint32_t tag, bool alive, uint4 (&r)[NB])
 {
     bool ok = false;
     for (uint32_t i = 0; i < kResWaitLimit; ++i) {
@@ -253,10 +256,7 @@ __device__ __forceinline__ void get_node_records(const uint4* q, int stride, uin
         }
         if (ok || !alive) break;
     }
-    if (!ok && alive) {
-        atomicOr(err, 1);
-        alive = false;
-    }
+    return ok;
 }
 
 // A node's stored state as 32-bit words: 9 populations, rho* and 8
@@ -472,7 +472,10 @@ __device__ __forceinline__ void run_resident(const Geom& g, const Phys& p, const
             const int2 hk = halo[k];
             const uint4* q = ex + hk.x;
             uint4 r[NB];
-            get_node_records(q, edge_cap, tag, err, alive, r);
+            if (!poll_records(q, edge_cap, tag, alive, r) && alive) {
+                atomicOr(err, 1);
+                alive = false;
+            }
             uint32_t v[NW];
             if constexpr (is16(ST)) {
                 v[0] = r[0].x; v[1] = r[0].y; v[2] = r[0].z; v[3] = r[NB - 1].x; v[4] = r[NB - 1].y;
