@@ -612,9 +612,10 @@ def time_to_steady_full(lbm, stream, cap=400000, check=1000):
     channels (width 32-256, length 512-2048, roughness 0-8, level 0-15, seed
     0) at full size, body force 1e-6, FP32 deviation storage; steady when
     |dQ|/|Q| < 1e-7 per 1000 steps, at most `cap` steps. Plain: each domain
-    run to steady alone (lbm_run_to_steady, 32-step CUDA graphs); batched: one
-    persistent launch per step over every domain not yet steady. Converged
-    and capped domains are reported apart."""
+    run to steady alone (lbm_run_to_steady: on the chip where it fits, else
+    32-step CUDA graphs); batched: every domain not yet steady, by one persistent
+    launch per step or in groups on the chip. Converged and capped domains are
+    reported apart."""
     import torch
     ws = batched_sweep()
     kw = dict(storage=lbm.LBM_FP32_DEV)

@@ -4,7 +4,8 @@
  * The library advances the lattice Boltzmann model of Li, Li, Chen & Fang,
  * "Lattice Boltzmann simulation of electrowetting-on-dielectric in a
  * rough-wall channel" (arXiv:0708.4182) on one GPU. One time step is one
- * fused CUDA kernel launch that performs, for every fluid node x:
+ * fused CUDA kernel (a launch per step, or many steps per launch for domains
+ * that fit on the chip; the same bits) that performs, for every fluid node x:
  *
  *   streaming      f_a(x, t) = f*_a(x - e_a, t-1), periodic in x and y,
  *                  half-way bounce-back where x - e_a is solid  (left side of Eq. 1)
@@ -204,10 +205,19 @@ lbm_status lbm_set_density_f32(lbm_ctx *ctx, const float *rho, int on_device);
  * Synchronises the context's stream when out is host memory. */
 lbm_status lbm_get_field(lbm_ctx *ctx, int which, double *out, int on_device);
 
-/* Advance nsteps >= 0 time steps (asynchronous). Runs of 32 plain steps
- * with no fused-observables step among them are replayed as one CUDA graph
- * (built on first use, per context). LBM_ESTATE before geometry and field
- * are set. */
+/* Advance nsteps >= 0 time steps (asynchronous). With the automatic thread
+ * layout and tile height (params.layout = LBM_LAYOUT_AUTO, tile_rows = 0), a
+ * domain that fits in the SMs' shared memory (about 0.6 M nodes at tau = 1, 0.3 M
+ * otherwise) runs its plain steps up to the next fused-observables step on the
+ * chip, many per launch of a cooperative kernel that holds its SMs for about
+ * three milliseconds at most; calls of one step (of two, for large domains) and
+ * calls under stream capture launch every step. Elsewhere runs of 32 plain steps
+ * are replayed as one CUDA graph (built on first use, per context). All ways give
+ * the same bits, and an even number of steps leaves the state in the same buffer
+ * of the workspace, so that a captured even number of steps stays valid between
+ * calls. All waits between CTAs on the device are bounded: one that gives up
+ * raises a flag, and the next call that reads back returns LBM_ETIMEOUT.
+ * LBM_ESTATE before geometry and field are set. */
 lbm_status lbm_step(lbm_ctx *ctx, int64_t nsteps);
 
 /* Launches of the resident kernel on this context so far (-1 for NULL): which
@@ -270,7 +280,8 @@ void lbm_destroy(lbm_ctx *ctx);
 
 /* ------------------------------------------------------------------------
  * Batches: many domains (different sizes, geometries and forces, one
- * storage form) advanced together, one persistent kernel launch per step.
+ * storage form) advanced together, one persistent kernel launch per step or
+ * many steps per launch where the domains fit on the chip.
  * Not in the paper, which runs its sweeps (over f and channel width) one
  * domain at a time; a batch runs such a sweep as one job.
  */
@@ -293,7 +304,10 @@ lbm_ctx *lbm_batch_domain(lbm_batch *b, int32_t i);
 
 /* Advance every active domain by nsteps. Each step is one launch of a
  * persistent kernel whose CTAs walk a tile list (domain, strip, row segment)
- * covering all active domains; pairs of steps run as one CUDA graph. */
+ * covering all active domains; pairs of steps run as one CUDA graph. Where every
+ * domain has the automatic layout and tile height and fits on the chip, and an
+ * estimate says that it is clearly faster (small domains), groups of domains run
+ * many steps per cooperative launch as in lbm_step; the bits are the same. */
 lbm_status lbm_batch_step(lbm_batch *b, int64_t nsteps);
 
 /* How count domains would be grouped to run on the chip (host arithmetic only, no

@@ -265,23 +265,23 @@ __host__ __device__ constexpr int conv_ntile(int n) { return n % 128 == 0 ? 128 
 // rings and 4 window slots were not faster. Measured on 16 images (us, before ->
 // now): 384 -> 128 channels at 16x64 66 -> 21, 128 -> 128 27 -> 12.5, 256 -> 256
 // at 8x32 46 -> 17, 192 -> 64 at 32x128 39 -> 35, 64 -> 192 49 -> 29, 96 -> 32 at
-// 64x256 56 -> 41, 32 -> 96 72 -> 39, 32 -> 32 30 -> 21. The sums run in the
+// 64x256 56 -> 41, 32 -> 96 72 -> 37, 32 -> 32 30 -> 21; on 8 images 96 -> 32 32 -> 24,
+// 32 -> 32 16.5 -> 14.4; on one, 32 -> 32 7.0 -> 7.2, 256 -> 256 43 -> 15. The sums run in the
 // order of the earlier kernels, so the outputs are the same bits.
 constexpr int kCvThreads = 256;
 constexpr int kCvProducers = kCvThreads - 64;
 constexpr int kWSlotsMax = 12;
-// weight taps per ring slot; window slots
+constexpr int kXSlots = 2;  // window slots
+// weight taps per ring slot
 template <int CK> __host__ __device__ constexpr int conv_tw() { return CK == 1 ? 3 : 1; }
-// window slots: a short group (few MMAs) needs more of them in flight
-template <int CK, int MT> __host__ __device__ constexpr int conv_xs() { return 2; }
 // window pixels for a strip of S columns, rounded up to 1 mod 8 so that the
 // planes of a pixel lie in different banks
 __host__ __device__ constexpr int conv_npx(int S, int mt) { return (128 * mt + 2 * (S + 2) + 2 + 6) / 8 * 8 + 1; }
 template <int NT, int NG, int CK> __host__ __device__ constexpr int conv_wbytes() { return conv_tw<CK>() * CK * NT * NG * 32; }
 template <int NT, int NG, int CK, int MT> __host__ __device__ constexpr size_t conv_smem(int S, int wslots)
 {
-    return size_t(conv_xs<CK, MT>()) * CK * conv_npx(S, MT) * 32 + size_t(wslots) * conv_wbytes<NT, NG, CK>() +
-           (2 * conv_xs<CK, MT>() + 2 * kWSlotsMax + 1) * 8 + 16 + size_t(conv_npx(S, MT)) * 4;
+    return size_t(kXSlots) * CK * conv_npx(S, MT) * 32 + size_t(wslots) * conv_wbytes<NT, NG, CK>() +
+           (2 * kXSlots + 2 * kWSlotsMax + 1) * 8 + 16 + size_t(conv_npx(S, MT)) * 4;
 }
 
 template <int NT, int NG, int CK, int MT>
@@ -294,7 +294,7 @@ __global__ void __launch_bounds__(kCvThreads) conv3x3_tc_kernel(const bf16* __re
     extern __shared__ __align__(1024) unsigned char smem[];
     constexpr int N = NT * NG;
     static_assert(MT * N <= 512, "the accumulators must fit the tensor memory");
-    constexpr int XS = conv_xs<CK, MT>(), TW = conv_tw<CK>();
+    constexpr int XS = kXSlots, TW = conv_tw<CK>();
     constexpr uint32_t kCols = tmem_cols(MT * N);
     constexpr int kWBytes = conv_wbytes<NT, NG, CK>();  // one weight slot: TW taps x CK chunks of N x 16
     const int npx = conv_npx(S, MT);
@@ -500,7 +500,7 @@ __global__ void __launch_bounds__(kCvThreads) conv3x3_tc_kernel(const bf16* __re
 // A thread takes the nine taps of one (n, k), which are contiguous in w, and
 // consecutive threads consecutive k, whose outputs lie in 16-byte runs (a thread
 // per output element found its place by 64-bit divisions and read 4 of every 36
-// bytes: 50 us for all layers of the network, now @PK@).
+// bytes: 50 us for all layers of the network, now 20).
 __device__ __forceinline__ void pack_pair(const float* __restrict__ w, int co, int ci, int transpose, int nt, int kc,
                                           int i, bf16* __restrict__ out)
 {
@@ -945,7 +945,7 @@ __global__ void head_bwd_kernel(const bf16* __restrict__ x, int ct, int Ci, cons
 // 32 or 64, views 16-byte aligned): the products of dx run in the same order;
 // the sums of dw and db go over the warp's lanes of one channel group by
 // shuffles, then over the warps. Memory bound; a channel a thread took 43 us for
-// 16 tiles of 64x256 and 32 channels, now @HB@.
+// 16 tiles of 64x256 and 32 channels, now 24.
 template <int CO>
 __global__ void __launch_bounds__(kT) head_bwd8_kernel(const bf16* __restrict__ x, int ct, int Ci,
                                                        const bf16* __restrict__ w, const float* __restrict__ dy, int HW,
@@ -1072,7 +1072,7 @@ __global__ void pool2_bwd_kernel(const bf16* __restrict__ dy, int cty, bf16* __r
 // 4 copies); a thread reads 8 channels (16 bytes) of a coarse pixel and writes
 // them four times, so C, ctx, cty must be multiples of 8 and the views 16-byte
 // aligned. (A thread per copy, placed by 64-bit divisions: 34 us for the three
-// upsamplings of 16 tiles of 64x256, now @UP@.)
+// upsamplings of 16 tiles of 64x256, now 19.)
 __global__ void up2_fwd_kernel(const bf16* __restrict__ x, int ctx, bf16* __restrict__ y, int cty, int C, int h,
                                int w, int B)
 {
@@ -1213,7 +1213,7 @@ __global__ void relu_bwd_kernel(const bf16* __restrict__ y, int cty, bf16* __res
 // FP32 NCHW planes -> BF16 NHWC with ct channels per pixel (channels >= c are
 // 0). V: a thread writes 8 channels of a pixel in 16 bytes (ct a multiple of 8,
 // y 16-byte aligned; an element a thread took 18 us for 16 tiles of 64x256, now
-// @IN@).
+// 5).
 template <bool V>
 __global__ void input_nhwc_kernel(const float* __restrict__ x, int C, int HW, int B, bf16* __restrict__ y, int ct)
 {

@@ -481,7 +481,8 @@ def lbm_batch_resident_plan(specs, edge_nodes: int = 0) -> list:
 
 
 class Batch:
-    """Many domains advanced together (one persistent launch per step).
+    """Many domains advanced together (one persistent launch per step, or many
+    steps per launch where the domains fit on the chip).
 
     ``specs`` is a list of dicts of ``make_params`` arguments (nx, ny and the
     model parameters of each domain; one storage form for all). ``domains``
